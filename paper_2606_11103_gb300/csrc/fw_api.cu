@@ -418,12 +418,50 @@ int make_dims(const fw_grid *g, int n_mech, int storage, bool nl, Dims *d)
     return FW_OK;
 }
 
-// per-class coefficient table for the run's dt (Eqs. relaxation_a/b), with
-// the midpoint memory-variable update folded in (ceff, hb); sc1 and sc2 scale
-// the stored memory variables of the gradient and divergence sides (binary16
-// storage).
-std::vector<double> build_lut(const std::vector<fw_relax_params> &cl, double dt, double sc1, double sc2)
+// Stored value of a memory variable = psi * scale.  binary16 storage keeps
+// psi in scaled units so that the memory variables of the expected fields
+// stay in the normal range of the format: the gradient side psi1 (Pa/m) is
+// stored as a pressure difference per cell in units of the reference
+// pressure p_ref (psi1 dx / p_ref), the divergence side psi2 (1/s) as the
+// same with the reference impedance rho c = 1.54e6 kg/(m^2 s)
+// (psi2 dx Z / p_ref).  p_ref follows the sources (fw_set_sources: 1/100 of
+// the largest pressure increment one step of the sources adds, about 1/100
+// of the emitted amplitude; 10 Pa before any source).  Other storages use 1.
+}  // namespace
+namespace fwgb {
+double psi_scale_of(const fw_medium *m, int side)
 {
+    if (m->storage != FW_STORE_F16) return 1.0;
+    const double pref = m->psi_pref, zref = 1000.0 * 1540.0;
+    return side == 1 ? m->dx / pref : m->dx * zref / pref;
+}
+}  // namespace fwgb
+namespace {
+
+// per-class coefficient table for the run's dt (Eqs. relaxation_a/b), with
+// the midpoint memory-variable update folded in (ceff, hb); the stored memory
+// variables of the gradient and divergence sides may be scaled (binary16
+// storage, psi_scale_of).
+// FP32 media: the sweeps take 1/kappa as a pair of FP32 values, and the pair
+// carries the correction for the FP32 rounding of dt (velocity side) and of the
+// stencil weights (their gain on long waves, both sides).  In a homogeneous
+// region such a rounding is the same in every cell, a coherent error of the
+// wave speed; uncorrected, 256 steps of a 256^2 plane ended 1.2e-6 to 2.5e-6
+// off the FP64 scheme.
+std::vector<double> build_lut(const fw_medium *m)
+{
+    const std::vector<fw_relax_params> &cl = m->classes;
+    const double dt = m->dt, sc1 = psi_scale_of(m, 1), sc2 = psi_scale_of(m, 2);
+    const bool f32 = m->es == 4;
+    double comp1 = 1.0, comp2 = 1.0;
+    if (f32) {
+        const double cm[4] = {1225.0 / 1024.0, -245.0 / 3072.0, 49.0 / 5120.0, -5.0 / 7168.0};
+        double gain = 0.0;   // sum over the rounded weights of (2k + 1) w_k dx, 1 without rounding
+        for (int k = 0; k < 4; ++k)
+            gain += (2 * k + 1) * double(float((m->time_order == 4 ? m->ts_a[k][0] : cm[k]) / m->dx)) * m->dx;
+        comp2 = 1.0 / gain;
+        comp1 = comp2 * dt / double(float(dt));
+    }
     std::vector<double> t(cl.size() * kLutStride, 0.0);
     for (size_t c = 0; c < cl.size(); ++c) {
         const fw_relax_params &p = cl[c];
@@ -449,24 +487,13 @@ std::vector<double> build_lut(const std::vector<fw_relax_params> &cl, double dt,
         e[3] = 1.0 / p.kappa2 + sa2;
         e[kLutDk] = sa1;
         e[kLutDk + 1] = sa2;
+        const double ik[2] = {comp1 / p.kappa1, comp2 / p.kappa2};
+        for (int k = 0; k < 2; ++k) {
+            e[kLutIk + k] = f32 ? double(float(ik[k])) : ik[k];
+            e[kLutIk + 2 + k] = ik[k] - e[kLutIk + k];
+        }
     }
     return t;
-}
-
-// Stored value of a memory variable = psi * scale.  binary16 storage keeps
-// psi in scaled units so that the memory variables of the expected fields
-// stay in the normal range of the format: the gradient side psi1 (Pa/m) is
-// stored as a pressure difference per cell in units of the reference
-// pressure p_ref (psi1 dx / p_ref), the divergence side psi2 (1/s) as the
-// same with the reference impedance rho c = 1.54e6 kg/(m^2 s)
-// (psi2 dx Z / p_ref).  p_ref follows the sources (fw_set_sources: 1/100 of
-// the largest pressure increment one step of the sources adds, about 1/100
-// of the emitted amplitude; 10 Pa before any source).  Other storages use 1.
-double psi_scale_of(const fw_medium *m, int side)
-{
-    if (m->storage != FW_STORE_F16) return 1.0;
-    const double pref = m->psi_pref, zref = 1000.0 * 1540.0;
-    return side == 1 ? m->dx / pref : m->dx * zref / pref;
 }
 
 template <typename T> std::vector<T> cast_vec(const std::vector<double> &v)
@@ -807,7 +834,7 @@ int create_common(const fw_grid *g, const float *c, const float *rho, const floa
         if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess) { release(m); return FW_ERR_CUDA; }
     }
     // class table and absorbing profiles
-    if ((rc = upload_doubles(m, m->lut, build_lut(classes, m->dt, psi_scale_of(m, 1), psi_scale_of(m, 2)), s))) { release(m); return rc; }
+    if ((rc = upload_doubles(m, m->lut, build_lut(m), s))) { release(m); return rc; }
     {
         const double r0 = g->pml_r0 > 0 ? g->pml_r0 : 1e-5;
         const double dmax = g->pml > 0 ? -3.0 * m->c_max * std::log(r0) / (2.0 * g->pml * g->dx) : 0.0;
@@ -852,7 +879,7 @@ int set_psi_reference(fw_medium *m, const float *waveforms, size_t wl)
     }
     FW_CK(cudaGetLastError());
     m->psi_pref = pref;
-    int rc = upload_doubles(m, m->lut, build_lut(m->classes, m->dt, psi_scale_of(m, 1), psi_scale_of(m, 2)), s);
+    int rc = upload_doubles(m, m->lut, build_lut(m), s);
     if (rc) return rc;
     FW_CK(cudaStreamSynchronize(s));
     return FW_OK;

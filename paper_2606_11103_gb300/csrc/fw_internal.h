@@ -29,11 +29,15 @@ int nelder_mead(int n, double *x, const double *lo, const double *hi,
                 double xatol, double fatol, double *fmin, int *n_iter, int *n_eval);
 
 // ---- device layout ---------------------------------------------------------
-constexpr int kLutStride = 32;   // values per class in the coefficient table
+constexpr int kLutStride = 36;   // values per class in the coefficient table
 // table block offsets (in values): 0 kappa1, 1 kappa2, 2 ceff1, 3 ceff2,
 // 4.. a1[4], 8.. b1[4], 12.. hb1[4], 16.. a2[4], 20.. b2[4], 24.. hb2[4],
-// 28 sum a1/2, 29 sum a2/2 (= ceff - 1/kappa, the part the layer ramp scales)
-constexpr int kLutA1 = 4, kLutB1 = 8, kLutH1 = 12, kLutA2 = 16, kLutB2 = 20, kLutH2 = 24, kLutDk = 28;
+// 28 sum a1/2, 29 sum a2/2 (= ceff - 1/kappa, the part the layer ramp scales),
+// 30 1/kappa1, 31 1/kappa2, 32, 33 what the rounding of 30, 31 left off (FP32
+// media; both with the known rounding of the global factors taken back, see
+// build_lut).  The sweeps use a, b and 30..33, the adjoint the others.
+constexpr int kLutA1 = 4, kLutB1 = 8, kLutH1 = 12, kLutA2 = 16, kLutB2 = 20, kLutH2 = 24, kLutDk = 28,
+              kLutIk = 30;
 
 struct Monitor {
     unsigned int max_bits;   // bits of max |p| (non-negative float)
@@ -75,6 +79,11 @@ struct Graph {
 };
 
 }  // namespace fwgb
+
+struct fw_medium;
+namespace fwgb {
+double psi_scale_of(const fw_medium *m, int side);   // stored memory variable = psi * scale (side 1 or 2)
+}
 
 struct fw_medium {
     fw_grid g{};

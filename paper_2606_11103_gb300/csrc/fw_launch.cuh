@@ -39,6 +39,8 @@ template <typename R> Geo<R> make_geo(const fw_medium *m)
     g.c3 = R(cm[2] / m->dx);
     g.c4 = R(cm[3] / m->dx);
     g.dt = R(m->dt);
+    g.hs1 = R(0.5 / psi_scale_of(m, 1));
+    g.hs2 = R(0.5 / psi_scale_of(m, 2));
     g.lr = R(m->g.transition > 0 ? m->g.transition : 0.5 * m->g.pml);
     for (int i = 0; i < 4; ++i)
         for (int n = 0; n < 4; ++n) g.ta[i][n] = R(m->ts_a[i][n] / m->dx);
