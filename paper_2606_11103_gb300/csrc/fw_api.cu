@@ -136,7 +136,7 @@ EncodeTiledFn tensor_map_encoder()
 void setup_tma(fw_medium *m)
 {
     m->tma = false;
-    if (m->ndim != 3 || m->storage == FW_STORE_F64) return;
+    if (m->storage == FW_STORE_F64) return;
     if (const char *e = std::getenv("FWGB_NO_TMA"))
         if (*e && *e != '0') return;
     EncodeTiledFn enc = tensor_map_encoder();
@@ -687,8 +687,7 @@ int choose_zseg(const fw_medium *m)
     // 16 planes per CTA measured best on the 512^3 workload (L2 sharing of
     // the halo planes between concurrently resident CTAs); at least 8 waves
     // of CTAs over the 152 SMs
-    const int tw = m->ndim == 3 ? (m->es == 8 ? 64 : 128) : 256;
-    const int by = m->ndim == 3 ? 8 : 1;
+    const int tw = m->es == 8 ? 64 : 128, by = 8;
     long long tiles = (long long)((m->NX + tw - 1) / tw) * ((m->NY + by - 1) / by);
     int z = 16;
     while (z > 8 && tiles * ((m->NZ + z - 1) / z) < 152LL * 8) z /= 2;

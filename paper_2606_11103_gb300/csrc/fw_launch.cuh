@@ -3,7 +3,9 @@
 // one translation unit per storage type so that they compile in parallel.
 #pragma once
 
-#include "fw_kernels.cuh"
+#include "fw_plane.cuh"
+
+#include <climits>
 
 #include <cuda.h>
 
@@ -20,7 +22,7 @@ namespace fwgb {
 template <typename R> struct Tile3 {
     static constexpr int BX = sizeof(R) == 8 ? 16 : 32, BYV = FWGB_VEL3_BY, BYP = FWGB_PRES3_BY;
 };
-template <typename R> struct Tile2 { static constexpr int BX = 64, BYV = 1, BYP = 1; };
+constexpr int kPlaneBY = 4;   // rows per CTA of the unstaged 2D sweeps
 
 template <typename R> Geo<R> make_geo(const fw_medium *m)
 {
@@ -49,10 +51,10 @@ template <typename R> Geo<R> make_geo(const fw_medium *m)
     return g;
 }
 
-// Tensor maps of the streams the 3D velocity sweep stages by TMA: every
-// array is addressed as a 3D tensor (px, NY, NZ) with the medium's pitches;
-// boxes are the CTA tile (TW x BY) or its halo boxes (p: (TW+8) x (BY+7)
-// from (xb-4, yb-3); rho: (TW+4) x (BY+1) from (xb, yb)).  Elements outside
+// Tensor maps of the streams that the sweeps stage by TMA: every array is
+// addressed as a 3D tensor (px, NY, NZ) with the medium's pitches; boxes are
+// the CTA tile (TW x BY along x and y, x and z in 2D) or its halo boxes (p:
+// (TW+8) x (BY+7) from (xb-4, yb-3); rho: (TW+4) x (BY+1)).  Elements outside
 // the tensor read as zero.  encode is the driver's tensor-map encoder.
 using EncodeTiledFn = CUresult (*)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
                                    const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
@@ -70,10 +72,39 @@ bool encode_map(EncodeTiledFn encode, TensorMapBlob *out, const fw_medium *m, co
 {
     const cuuint64_t dims[3] = {(cuuint64_t)m->px, (cuuint64_t)m->NY, (cuuint64_t)m->NZ};
     const cuuint64_t strides[2] = {(cuuint64_t)m->px * sizeof(T), (cuuint64_t)m->plane * sizeof(T)};
-    const cuuint32_t box[3] = {bx, by, 1}, estr[3] = {1, 1, 1};
+    const cuuint32_t box[3] = {bx, m->ndim == 3 ? by : 1, m->ndim == 3 ? 1 : by}, estr[3] = {1, 1, 1};
     return encode(reinterpret_cast<CUtensorMap *>(out), map_type<T>(), 3, const_cast<void *>(base), dims, strides,
                   box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
                   CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// 2D tiles (k_velocity_tiles, k_pressure_tiles)
+template <typename SS, typename SP> bool build_plane_maps(EncodeTiledFn encode, fw_medium *m)
+{
+    constexpr unsigned W = kTileW, H = kTileH;
+    const bool ts = m->time_order == 4;
+    VelMaps &v = m->vel_maps;
+    PresMaps &q = m->pres_maps;
+    bool ok = encode_map<SS>(encode, &v.p_halo, m, m->p, W + 8, H + 7) &&
+              encode_map<SS>(encode, &v.rho_halo, m, m->rho, W + 4, H + 1) &&
+              encode_map<uint16_t>(encode, &v.cls, m, m->cls, W, H) && encode_map<SS>(encode, &v.kdt, m, m->kdt, W, H);
+    q.cls = v.cls;
+    q.kdt = v.kdt;
+    for (int ax = 0; ax < 3; ax += 2) {
+        ok = ok && encode_map<SS>(encode, &v.v[ax], m, m->v[ax], W, H);
+        for (int n = 0; n < m->nmech; ++n) ok = ok && encode_map<SP>(encode, &v.psi[n][ax], m, m->psi1[n][ax], W, H);
+    }
+    for (int n = 0; n < m->nmech; ++n) ok = ok && encode_map<SP>(encode, &q.psi[n], m, m->psi2[n], W, H);
+    ok = ok && encode_map<SS>(encode, &q.p_own, m, m->p, W, H) &&
+         (!m->nonlinear || encode_map<SS>(encode, &q.b2dt, m, m->b2dt, W, H));
+    if (ts)
+        ok = ok && encode_map<SS>(encode, &q.vx_ring, m, m->v[0], W + 8, H + 2) &&
+             encode_map<SS>(encode, &q.vz_ring, m, m->v[2], W + 8, H + 7) &&
+             encode_map<SS>(encode, &q.rho_own, m, m->rho, W, H);
+    else
+        ok = ok && encode_map<SS>(encode, &q.vx_halo, m, m->v[0], W + 8, H) &&
+             encode_map<SS>(encode, &q.vz_own, m, m->v[2], W, H + 7);
+    return ok;
 }
 
 template <typename R, typename SS, typename SP>
@@ -82,6 +113,7 @@ bool build_vel_maps_t(EncodeTiledFn encode, fw_medium *m)
     if constexpr (sizeof(R) != 4) {
         return false;
     } else {
+        if (m->ndim == 2) return build_plane_maps<SS, SP>(encode, m);
         constexpr int TW = 4 * Tile3<R>::BX, BY = Tile3<R>::BYV;
         VelMaps &v = m->vel_maps;
         bool ok = encode_map<SS>(encode, &v.p_halo, m, m->p, TW + 8, BY + 7) &&
@@ -114,122 +146,168 @@ bool build_vel_maps_t(EncodeTiledFn encode, fw_medium *m)
     }
 }
 
-// which: bit 0 = velocity sweep, bit 1 = pressure sweep, bit 2 = only opt the
-// instances into their dynamic shared memory (done once at medium creation,
-// outside any stream capture).  im (may be null): a step from one state
-// image into another (StepImages) instead of the in-place step of the
-// medium's own state.
-template <typename R, typename SS, typename SP, int DIM, int NM, bool TS>
-cudaError_t launch_dn(const fw_medium *m, cudaStream_t s, int which, const StepImages *im)
-{
-    constexpr int BX = DIM == 3 ? Tile3<R>::BX : Tile2<R>::BX;
-    constexpr int BYV = DIM == 3 ? Tile3<R>::BYV : Tile2<R>::BYV;
-    constexpr int BYP = DIM == 3 ? Tile3<R>::BYP : Tile2<R>::BYP;
-    // the 3D FP32-state velocity sweep stages its streams by TMA when the
-    // medium holds tensor maps for them (the cp.async instance otherwise)
-    constexpr bool CAN_TMA = DIM == 3 && sizeof(R) == 4;
-    using LV = VelSmem<R, SS, SP, DIM, NM, BX, BYV, TS>;
-    using LVT = VelSmem<R, SS, SP, DIM, NM, BX, BYV, TS, CAN_TMA>;
-    using LP = PresSmem<R, SS, SP, DIM, NM, BX, BYP, TS>;
-    using LPT = PresSmem<R, SS, SP, DIM, NM, BX, BYP, TS, CAN_TMA>;
-    if (which & 4) {
-        cudaError_t e = cudaFuncSetAttribute(k_velocity<R, SS, SP, DIM, NM, BX, BYV, TS, false>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LV::bytes);
-        if constexpr (CAN_TMA)
-            if (e == cudaSuccess)
-                e = cudaFuncSetAttribute(k_velocity<R, SS, SP, DIM, NM, BX, BYV, TS, true>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LVT::bytes);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k_pressure<R, SS, SP, DIM, NM, BX, BYP, true, TS, false>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LP::bytes);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k_pressure<R, SS, SP, DIM, NM, BX, BYP, false, TS, false>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LP::bytes);
-        if constexpr (CAN_TMA) {
-            if (e == cudaSuccess)
-                e = cudaFuncSetAttribute(k_pressure<R, SS, SP, DIM, NM, BX, BYP, true, TS, true>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LPT::bytes);
-            if (e == cudaSuccess)
-                e = cudaFuncSetAttribute(k_pressure<R, SS, SP, DIM, NM, BX, BYP, false, TS, true>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LPT::bytes);
-        }
-        return e;
-    }
-    const Geo<R> g = make_geo<R>(m);
-    const int gx = (m->NX + 4 * BX - 1) / (4 * BX), gz = (m->NZ + m->zseg - 1) / m->zseg;
-    // a state array of the medium, or the same array in the image read (rd)
-    // or written (nw) by an image step
-    const char *slab = static_cast<const char *>(m->slab);
-    auto rd = [&](void *a) -> void * {
+// A state array of the medium, or the same array in the image read (rd) or
+// written (nw) by an image step
+struct StateAt {
+    const char *slab;
+    const StepImages *im;
+    void *rd(void *a) const
+    {
         return (a && im) ? const_cast<char *>(im->rd) + (static_cast<const char *>(a) - slab) : a;
-    };
-    auto nw = [&](void *a) -> void * { return (a && im) ? static_cast<char *>(rd(a)) + im->wofs : a; };
-    const long long wofs = im ? im->wofs : 0;
-    const bool tma = m->tma && !im;   // tensor maps address the medium's own arrays
+    }
+    void *nw(void *a) const { return (a && im) ? static_cast<char *>(rd(a)) + im->wofs : a; }
+};
 
+template <typename R, typename SS, typename SP, int NM>
+VelArgs<R, SS, SP> vel_args(const fw_medium *m, const StepImages *im)
+{
+    const StateAt at{static_cast<const char *>(m->slab), im};
     VelArgs<R, SS, SP> va{};
-    va.g = g;
-    va.p = static_cast<const SS *>(rd(m->p));
-    va.wofs = wofs;
+    va.g = make_geo<R>(m);
+    va.p = static_cast<const SS *>(at.rd(m->p));
+    va.wofs = im ? im->wofs : 0;
     for (int ax = 0; ax < 3; ++ax) {
-        va.v[ax] = static_cast<SS *>(rd(m->v[ax]));
-        va.psip[ax] = static_cast<SS *>(rd(m->psi1p[ax]));
+        va.v[ax] = static_cast<SS *>(at.rd(m->v[ax]));
+        va.psip[ax] = static_cast<SS *>(at.rd(m->psi1p[ax]));
         va.pd[ax] = static_cast<const R *>(m->prof[ax][0]);
         va.pa[ax] = static_cast<const R *>(m->prof[ax][1]);
-        for (int n = 0; n < NM; ++n) va.psi[n][ax] = static_cast<SP *>(rd(m->psi1[n][ax]));
+        for (int n = 0; n < NM; ++n) va.psi[n][ax] = static_cast<SP *>(at.rd(m->psi1[n][ax]));
     }
     va.rho = static_cast<const SS *>(m->rho);
     va.cls = m->cls;
     va.lut = static_cast<const R *>(m->lut);
     va.kdt = static_cast<const SS *>(m->kdt);
     va.mon = m->mon;
-    if (which & 1) {
-        const dim3 gv(gx, (m->NY + BYV - 1) / BYV, gz), bv(BX, BYV);
-        bool done = false;
-        if constexpr (CAN_TMA) {
-            if (tma) {
-                va.maps = m->vel_maps;
-                k_velocity<R, SS, SP, DIM, NM, BX, BYV, TS, true><<<gv, bv, LVT::bytes, s>>>(va);
-                done = true;
-            }
-        }
-        if (!done) k_velocity<R, SS, SP, DIM, NM, BX, BYV, TS, false><<<gv, bv, LV::bytes, s>>>(va);
-    }
-    if (!(which & 2)) return cudaGetLastError();
+    return va;
+}
 
+template <typename R, typename SS, typename SP, int NM>
+PresArgs<R, SS, SP> pres_args(const fw_medium *m, const StepImages *im)
+{
+    const StateAt at{static_cast<const char *>(m->slab), im};
     PresArgs<R, SS, SP> pa{};
-    pa.g = g;
-    pa.p = static_cast<SS *>(rd(m->p));
-    pa.wofs = wofs;
+    pa.g = make_geo<R>(m);
+    pa.p = static_cast<SS *>(at.rd(m->p));
+    pa.wofs = im ? im->wofs : 0;
     for (int ax = 0; ax < 3; ++ax) {
-        pa.v[ax] = static_cast<const SS *>(nw(m->v[ax]));   // this step's velocity
-        pa.psip[ax] = static_cast<SS *>(rd(m->psi2p[ax]));
+        pa.v[ax] = static_cast<const SS *>(at.nw(m->v[ax]));   // this step's velocity
+        pa.psip[ax] = static_cast<SS *>(at.rd(m->psi2p[ax]));
         pa.pd[ax] = static_cast<const R *>(m->prof[ax][2]);
         pa.pa[ax] = static_cast<const R *>(m->prof[ax][3]);
     }
-    for (int n = 0; n < NM; ++n) pa.psi[n] = static_cast<SP *>(rd(m->psi2[n]));
+    for (int n = 0; n < NM; ++n) pa.psi[n] = static_cast<SP *>(at.rd(m->psi2[n]));
     pa.kdt = static_cast<const SS *>(m->kdt);
     pa.b2dt = static_cast<const SS *>(m->b2dt);
     pa.cls = m->cls;
     pa.lut = static_cast<const R *>(m->lut);
     pa.mon = m->mon;
     pa.rho = static_cast<const SS *>(m->rho);
-    const dim3 gp(gx, (m->NY + BYP - 1) / BYP, gz), bp(BX, BYP);
-    if constexpr (CAN_TMA) {
-        if (tma) {
-            pa.maps = m->pres_maps;
-            if (m->nonlinear)
-                k_pressure<R, SS, SP, DIM, NM, BX, BYP, true, TS, true><<<gp, bp, LPT::bytes, s>>>(pa);
-            else
-                k_pressure<R, SS, SP, DIM, NM, BX, BYP, false, TS, true><<<gp, bp, LPT::bytes, s>>>(pa);
-            return cudaGetLastError();
+    return pa;
+}
+
+// Sweeps of one dimension, mechanism count and time scheme.  which: bit 0 =
+// velocity sweep, bit 1 = pressure sweep, bit 2 = only opt the instances into
+// their dynamic shared memory (done once at medium creation, outside any
+// stream capture).  im (may be null): a step from one state image into another
+// (StepImages) instead of the in-place step of the medium's own state.
+// 2D FP32-state grids from kTileMin tiles on take the staged sweeps, in runs of
+// two tiles per CTA, of four from kTileLong tiles on; smaller grids, FP64 media
+// and image steps the unstaged ones.  Measured, us per step (unstaged / staged
+// in runs of 1, 2, 4, 8; N = 4, FP32): 512^2 (512 tiles) 10.7 / 13.1, 13.9,
+// 20.1, 32.3; 1024^2 (2048) 28.3 / 30.7, 27.6, 31.5, 38.9; 2048^2 (8192) 116 /
+// 114, 102, 104, 110; 4096^2 (32768) 431 / 415, 373, 363, 373.  A run hides
+// the latency of a tile's copies behind the tile before it, a short one leaves
+// the hardware more CTAs to balance: with one persistent CTA per slot and even
+// shares the 4096^2 step took 439 us, its slowest SMs finishing last.
+constexpr int kTileMin = 2048, kTileLong = 16384;
+
+template <typename SP, int NM, bool TS>
+cudaError_t launch_tiles(const fw_medium *m, cudaStream_t s, int which, int gx, int n_tiles)
+{
+    constexpr int NS = 2;   // stages: the tile computed and the one on its way
+    using LV = VelTile<SP, NM, TS>;
+    const size_t bv = NS * LV::stage + 8 * NS;
+    const size_t bp = NS * (m->nonlinear ? PresTile<SP, NM, true, TS>::stage : PresTile<SP, NM, false, TS>::stage) + 8 * NS;
+    const auto kv = k_velocity_tiles<SP, NM, TS, NS>;
+    const auto kp = m->nonlinear ? k_pressure_tiles<SP, NM, true, TS, NS> : k_pressure_tiles<SP, NM, false, TS, NS>;
+    if (which & 4) {
+        const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+        const cudaError_t e = cudaFuncSetAttribute(kv, attr, (int)bv);
+        return e == cudaSuccess ? cudaFuncSetAttribute(kp, attr, (int)bp) : e;
+    }
+    const dim3 block(32, kTileH);
+    const int run = n_tiles >= kTileLong ? 4 : 2;
+    const int rows = n_tiles / gx, ctas = gx * ((rows + run - 1) / run);
+    if (which & 1) kv<<<ctas, block, bv, s>>>(vel_args<float, float, SP, NM>(m, nullptr), m->vel_maps, gx, run, rows);
+    if (which & 2) kp<<<ctas, block, bp, s>>>(pres_args<float, float, SP, NM>(m, nullptr), m->pres_maps, gx, run, rows);
+    return cudaGetLastError();
+}
+
+template <typename R, typename SS, typename SP, int NM, bool TS>
+cudaError_t launch_2d(const fw_medium *m, cudaStream_t s, int which, const StepImages *im)
+{
+    const int gx = (m->NX + 127) / 128;
+    if constexpr (sizeof(R) == 4) {
+        const long long n_tiles = (long long)gx * ((m->NZ + kTileH - 1) / kTileH);
+        if (which & 4) return launch_tiles<SP, NM, TS>(m, s, which, gx, 0);
+        if (m->tma && !im && n_tiles >= kTileMin && n_tiles < INT_MAX) return launch_tiles<SP, NM, TS>(m, s, which, gx, (int)n_tiles);
+    }
+    if (which & 4) return cudaSuccess;
+    const dim3 grid((unsigned)gx * (unsigned)((m->NZ + kPlaneBY - 1) / kPlaneBY)), block(32, kPlaneBY);
+    if (which & 1) k_velocity_plane<R, SS, SP, NM, kPlaneBY, TS><<<grid, block, 0, s>>>(vel_args<R, SS, SP, NM>(m, im), gx);
+    if (which & 2) {
+        const auto pa = pres_args<R, SS, SP, NM>(m, im);
+        if (m->nonlinear) k_pressure_plane<R, SS, SP, NM, kPlaneBY, true, TS><<<grid, block, 0, s>>>(pa, gx);
+        else k_pressure_plane<R, SS, SP, NM, kPlaneBY, false, TS><<<grid, block, 0, s>>>(pa, gx);
+    }
+    return cudaGetLastError();
+}
+
+template <typename R, typename SS, typename SP, int NM, bool TS, bool TMA>
+cudaError_t launch_3d_as(const fw_medium *m, cudaStream_t s, int which, const StepImages *im)
+{
+    constexpr int BX = Tile3<R>::BX, BYV = Tile3<R>::BYV, BYP = Tile3<R>::BYP;
+    using LV = VelSmem<R, SS, SP, NM, BX, BYV, TS, TMA>;
+    using LP = PresSmem<R, SS, SP, NM, BX, BYP, TS, TMA>;
+    const auto kv = k_velocity<R, SS, SP, NM, BX, BYV, TS, TMA>;
+    const auto kp = k_pressure<R, SS, SP, NM, BX, BYP, false, TS, TMA>, kpn = k_pressure<R, SS, SP, NM, BX, BYP, true, TS, TMA>;
+    if (which & 4) {
+        const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+        cudaError_t e = cudaFuncSetAttribute(kv, attr, (int)LV::bytes);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(kp, attr, (int)LP::bytes);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(kpn, attr, (int)LP::bytes);
+        return e;
+    }
+    MapsArg<TMA, VelMaps> vm;
+    MapsArg<TMA, PresMaps> pm;
+    if constexpr (TMA) {
+        vm = m->vel_maps;
+        pm = m->pres_maps;
+    }
+    const int gx = (m->NX + 4 * BX - 1) / (4 * BX), gz = (m->NZ + m->zseg - 1) / m->zseg;
+    if (which & 1)
+        kv<<<dim3(gx, (m->NY + BYV - 1) / BYV, gz), dim3(BX, BYV), LV::bytes, s>>>(vel_args<R, SS, SP, NM>(m, im), vm);
+    if (which & 2)
+        (m->nonlinear ? kpn : kp)<<<dim3(gx, (m->NY + BYP - 1) / BYP, gz), dim3(BX, BYP), LP::bytes, s>>>(
+            pres_args<R, SS, SP, NM>(m, im), pm);
+    return cudaGetLastError();
+}
+
+// The FP32-state sweeps stage their streams by TMA when the medium holds
+// tensor maps for them (which address the medium's own arrays, so not for
+// image steps), by cp.async otherwise.
+template <typename R, typename SS, typename SP, int NM, bool TS>
+cudaError_t launch_3d(const fw_medium *m, cudaStream_t s, int which, const StepImages *im)
+{
+    if constexpr (sizeof(R) == 4) {
+        if (which & 4) {
+            const cudaError_t e = launch_3d_as<R, SS, SP, NM, TS, true>(m, s, which, im);
+            if (e != cudaSuccess) return e;
+        } else if (m->tma && !im) {
+            return launch_3d_as<R, SS, SP, NM, TS, true>(m, s, which, im);
         }
     }
-    if (m->nonlinear)
-        k_pressure<R, SS, SP, DIM, NM, BX, BYP, true, TS, false><<<gp, bp, LP::bytes, s>>>(pa);
-    else
-        k_pressure<R, SS, SP, DIM, NM, BX, BYP, false, TS, false><<<gp, bp, LP::bytes, s>>>(pa);
-    return cudaGetLastError();
+    return launch_3d_as<R, SS, SP, NM, TS, false>(m, s, which, im);
 }
 
 template <typename R, typename SS, typename SP, bool TS>
@@ -237,10 +315,10 @@ cudaError_t launch_ts(const fw_medium *m, cudaStream_t s, int which, const StepI
 {
     const bool d3 = m->ndim == 3;
     switch (m->nmech) {
-    case 1: return d3 ? launch_dn<R, SS, SP, 3, 1, TS>(m, s, which, im) : launch_dn<R, SS, SP, 2, 1, TS>(m, s, which, im);
-    case 2: return d3 ? launch_dn<R, SS, SP, 3, 2, TS>(m, s, which, im) : launch_dn<R, SS, SP, 2, 2, TS>(m, s, which, im);
-    case 3: return d3 ? launch_dn<R, SS, SP, 3, 3, TS>(m, s, which, im) : launch_dn<R, SS, SP, 2, 3, TS>(m, s, which, im);
-    case 4: return d3 ? launch_dn<R, SS, SP, 3, 4, TS>(m, s, which, im) : launch_dn<R, SS, SP, 2, 4, TS>(m, s, which, im);
+    case 1: return d3 ? launch_3d<R, SS, SP, 1, TS>(m, s, which, im) : launch_2d<R, SS, SP, 1, TS>(m, s, which, im);
+    case 2: return d3 ? launch_3d<R, SS, SP, 2, TS>(m, s, which, im) : launch_2d<R, SS, SP, 2, TS>(m, s, which, im);
+    case 3: return d3 ? launch_3d<R, SS, SP, 3, TS>(m, s, which, im) : launch_2d<R, SS, SP, 3, TS>(m, s, which, im);
+    case 4: return d3 ? launch_3d<R, SS, SP, 4, TS>(m, s, which, im) : launch_2d<R, SS, SP, 4, TS>(m, s, which, im);
     default: return cudaErrorInvalidValue;
     }
 }
