@@ -14,19 +14,20 @@
 //
 // The adjoint of one time step is reverse-mode differentiation of the two
 // sweeps of fw_kernels.cuh, in the kernels' own variables (memory variables
-// of the divergence side summed over directions, midpoint update folded into
-// ceff and hb = (1 + b)/2):
-//   pressure: stp = ceff2 div + sum hb2 psi2 + absorbing, psi2' = b2 psi2 + a2 div,
-//             p' = p - K dt stp,  div = sum_d D-_d v_d;
-//   velocity: st = ceff1 g + sum hb1 psi1 + absorbing, psi1' = b1 psi1 + a1 g,
-//             v' = v - dtr st,  g = D+_d p;
-// (in the absorbing layer a -> r a and ceff -> 1/kappa + r (ceff - 1/kappa),
-// r the tissue ramp of the cell);
+// of the divergence side summed over directions; r the tissue ramp of the cell,
+// 1 outside the absorbing layer):
+//   pressure: psi2' = b2 psi2 + r a2 div, stp = div/kappa2 + sum (psi2 + psi2')/2
+//             + absorbing, p' = p - K dt stp,  div = sum_d D-_d v_d;
+//   velocity: psi1' = b1 psi1 + r a1 g, st = g/kappa1 + sum (psi1 + psi1')/2
+//             + absorbing, v' = v - dtr st,  g = D+_d p;
 // with (D+)^T = -D- and (D-)^T = -D+ for zero values beyond the grid.
-// A reverse step is receiver injection and the source-gain gradient, then the
-// pressure adjoint (pointwise; gives the adjoint of q_d), the velocity adjoint
-// (a stencil of that, pointwise; gives the adjoint of g_d) and the stencil
-// update of the pressure adjoint: one tiled kernel in 2D, three kernels in 3D.
+// A reverse step is two kernels, one thread per quad of four x points, every
+// operand read straight from memory:
+//   k_adj_pressure: the update of the pressure adjoint by the later step's
+//       adjoint of g_d (-D-), then the pressure adjoint (gives that of q_d);
+//   k_adj_velocity: the velocity adjoint (a stencil of the adjoint of q_d;
+//       gives that of g_d);
+// and between them k_adj_io, the transpose of injection and recording.
 // Gradients accumulate in FP64.
 // The linear system only (no nonlinear factor); FP32 and FP64 media.
 #include "fw_internal.h"
@@ -34,7 +35,6 @@
 
 #include <algorithm>
 #include <cmath>
-#include <utility>
 #include <vector>
 
 namespace fwgb {
@@ -57,15 +57,12 @@ template <typename R> struct AdjState {
 };
 
 template <typename R> struct AdjArgs {
-    int nx, ny, nz, px, nmech;
-    long long plane, vol;
-    bool ax_on[3];
+    int nx, ny, nz, px;
+    long long plane;
     R c1, c2, c3, c4, dt;
     int wabs;          // absorbing width (0: none) and 1 / length of the tissue ramp
     R inv_lr;
-    // adjoint state after the step (read) and before it (written; the same buffer
-    // for the three-kernel form, the other buffer of a pair for the one-kernel form)
-    AdjState<R> in, out;
+    AdjState<R> L;     // adjoint state, updated in place from after the step to before it
     // forward state before the step (f) and velocity after it (fv1)
     const R *fp, *fpsi1[kMaxMech][3], *fpsi2[kMaxMech], *fpsi2p[3];
     const R *fv1[3];
@@ -74,246 +71,291 @@ template <typename R> struct AdjArgs {
     const uint16_t *cls;
     const R *lut, *dlut;
     const R *pdh[3], *pah[3], *pdi[3], *pai[3];   // absorbing profile at half / integer points
-    // scratch of the three-kernel form: adjoints of q_d and of g_d
-    R *Q[3], *Gd[3];
+    R *Q[3], *Gd[3];   // adjoints of q_d (this step) and of g_d (the later step, then this one)
+    R *gsp;            // this step's pressure-side term of the gradient with respect to the d factor
     double *gk, *gs;
 };
 
-template <typename R> struct Pt {
-    int c[3];          // coordinate along each kernel axis
-    int n[3];          // axis lengths
-    long long st[3];   // strides
+// A thread's quad: coordinates, row lengths and strides per kernel axis
+struct AdjPos {
+    int c[3], n[3];
+    long long st[3], i;
+    bool on;
 };
 
-template <typename R>
-__device__ __forceinline__ Pt<R> make_pt(const AdjArgs<R> &A, int x, int y, int z)
+constexpr int kAdjRows = 4;   // rows of quads per CTA (y in 3D, depth in 2D)
+
+template <typename R, int DIM> __device__ __forceinline__ AdjPos adj_pos(const AdjArgs<R> &A)
 {
-    Pt<R> p;
-    p.c[0] = x; p.c[1] = y; p.c[2] = z;
-    p.n[0] = A.nx; p.n[1] = A.ny; p.n[2] = A.nz;
-    p.st[0] = 1; p.st[1] = A.px; p.st[2] = A.plane;
-    return p;
+    const unsigned gx = (unsigned)(A.nx + 127) / 128;
+    unsigned r = blockIdx.x / gx;
+    AdjPos P;
+    P.c[0] = 4 * (int)((blockIdx.x % gx) * 32 + threadIdx.x);
+    if (DIM == 3) {
+        const unsigned gy = (unsigned)(A.ny + kAdjRows - 1) / kAdjRows;
+        P.c[1] = (int)(r % gy) * kAdjRows + threadIdx.y;
+        P.c[2] = (int)(r / gy);
+    } else {
+        P.c[1] = 0;
+        P.c[2] = (int)r * kAdjRows + threadIdx.y;
+    }
+    P.n[0] = A.nx; P.n[1] = A.ny; P.n[2] = A.nz;
+    P.st[0] = 1; P.st[1] = A.px; P.st[2] = A.plane;
+    P.on = P.c[0] < A.nx && P.c[1] < A.ny && P.c[2] < A.nz;
+    P.i = (long long)P.c[2] * A.plane + (long long)P.c[1] * A.px + P.c[0];
+    return P;
 }
 
-// One thread per point: x from the block's x range and thread, the other two
-// kernel axes from the grid's y and z (no division of a flat index).
-template <typename R>
-__device__ __forceinline__ bool point(const AdjArgs<R> &A, Pt<R> &p, long long &i)
+// staggered difference of f along axis ax at the quad's cells, zero beyond the
+// grid: forward (at + 1/2) or backward
+template <typename R, int ax, bool FORWARD>
+__device__ __forceinline__ void adj_diff(const AdjArgs<R> &A, const AdjPos &P, const R *f, R (&out)[4])
 {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    if (x >= A.nx) return false;
-    p = make_pt(A, x, (int)blockIdx.y, (int)blockIdx.z);
-    i = (long long)blockIdx.z * A.plane + (long long)blockIdx.y * A.px + x;
-    return true;
+    if (ax == 0) {
+        R w[12], t[4];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const int x = P.c[0] + 4 * (k - 1);
+            ld4_or_zero(f + P.i + 4 * (k - 1), x >= 0 && x < A.px, t);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) w[4 * k + e] = t[e];
+        }
+        quad_diff_x(A, w, FORWARD ? 5 : 4, out);
+    } else {
+        R t[8][4];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const int d = j - (FORWARD ? 3 : 4), c = P.c[ax] + d;
+            ld4_or_zero(f + P.i + d * P.st[ax], c >= 0 && c < P.n[ax], t[j]);
+        }
+        quad_diff(A, t, out);
+    }
 }
 
-// forward staggered derivative at c + 1/2: sum_m c_m (f[c+m] - f[c-m+1])
-template <typename R>
-__device__ __forceinline__ R dplus(const AdjArgs<R> &A, const R *f, long long i, int c, int n, long long st)
-{
-    auto at = [&](int cc) -> R { return (cc >= 0 && cc < n) ? __ldg(f + i + (long long)(cc - c) * st) : R(0); };
-    return A.c1 * (at(c + 1) - at(c)) + A.c2 * (at(c + 2) - at(c - 1)) + A.c3 * (at(c + 3) - at(c - 2)) +
-           A.c4 * (at(c + 4) - at(c - 3));
-}
+// coefficients of one cell: 1/kappa (two parts), a, b and their derivatives by
+// the factor on d
+template <typename R, int NM> struct CellCoef {
+    R ik, il, a[4], b[4], da[4], db[4];
+    __device__ __forceinline__ void load(const AdjArgs<R> &A, int cls, int side)
+    {
+        lut2(A.lut, cls, side == 1 ? kLutIk1 : kLutIk2, ik, il);
+        lut4(A.lut, cls, side == 1 ? kLutA1 : kLutA2, a);
+        lut4(A.lut, cls, side == 1 ? kLutB1 : kLutB2, b);
+        const R *d = A.dlut + (size_t)cls * kDStride + (side == 1 ? 0 : 8);
+        Io<R>::ldg(d, da);
+        Io<R>::ldg(d + 4, db);
+    }
+};
 
-// backward staggered derivative at c of a half-point field: sum_m c_m (f[c+m-1] - f[c-m])
+// tissue-mechanism strength of the cell e of the quad (the forward sweeps' ramp)
 template <typename R>
-__device__ __forceinline__ R dminus(const AdjArgs<R> &A, const R *f, long long i, int c, int n, long long st)
+__device__ __forceinline__ R adj_ramp(const AdjArgs<R> &A, const AdjPos &P, int e)
 {
-    auto at = [&](int cc) -> R { return (cc >= 0 && cc < n) ? __ldg(f + i + (long long)(cc - c) * st) : R(0); };
-    return A.c1 * (at(c) - at(c - 1)) + A.c2 * (at(c + 1) - at(c - 2)) + A.c3 * (at(c + 2) - at(c - 3)) +
-           A.c4 * (at(c + 3) - at(c - 4));
-}
-
-// the same two differences of a run of values in shared memory (f[k] at the point + k,
-// zero beyond the grid already stored)
-template <typename R>
-__device__ __forceinline__ R dplus_s(const AdjArgs<R> &A, const R *f, int st)
-{
-    return A.c1 * (f[st] - f[0]) + A.c2 * (f[2 * st] - f[-st]) + A.c3 * (f[3 * st] - f[-2 * st]) +
-           A.c4 * (f[4 * st] - f[-3 * st]);
-}
-
-template <typename R>
-__device__ __forceinline__ R dminus_s(const AdjArgs<R> &A, const R *f, int st)
-{
-    return A.c1 * (f[0] - f[-st]) + A.c2 * (f[st] - f[-2 * st]) + A.c3 * (f[2 * st] - f[-3 * st]) +
-           A.c4 * (f[3 * st] - f[-4 * st]);
-}
-
-// tissue-mechanism strength of the cell (the forward sweeps' ramp, same arithmetic)
-template <typename R>
-__device__ __forceinline__ R cell_ramp(const AdjArgs<R> &A, const Pt<R> &P)
-{
-    if (A.wabs <= 0) return R(1);
-    const R s = fmax(fmax(layer_depth<R>(P.c[0], A.nx, A.wabs), layer_depth<R>(P.c[1], A.ny, A.wabs)),
+    const R s = fmax(fmax(layer_depth<R>(P.c[0] + e, A.nx, A.wabs), layer_depth<R>(P.c[1], A.ny, A.wabs)),
                      layer_depth<R>(P.c[2], A.nz, A.wabs));
     return ramp_of(s, A.inv_lr);
 }
 
-// Pressure adjoint at an in-grid point i: the adjoints of q_d (Qv).  FULL also
-// takes the gradient terms of the step (gs, gk) and writes the memory
-// variables before the step; without FULL only the adjoint state is read
-// (the halo of the one-kernel form).
-template <typename R, int DIM, int NM, bool FULL>
-__device__ __forceinline__ void pres_point(const AdjArgs<R> &A, const Pt<R> &P, long long i, R (&Qv)[3], R &gs,
-                                           double &gk)
+template <typename R, int DIM> __device__ __forceinline__ bool adj_in_layer(const AdjArgs<R> &A, const AdjPos &P, int ax)
 {
-    const int cl = __ldg(A.cls + i);
-    const R *t = A.lut + (size_t)cl * kLutStride;
-    const R *dtb = A.dlut + (size_t)cl * kDStride;
-    R q[3] = {0, 0, 0}, div = 0;
-    if (FULL) {
+    if (A.wabs <= 0 || (DIM == 2 && ax == 1)) return false;
+    const int c = P.c[ax], last = ax == 0 ? c + 3 : c;
+    return c < A.wabs || last >= P.n[ax] - A.wabs;
+}
+
+__device__ __forceinline__ void add4(double *p, const double (&v)[4])
+{
+    double2 *q = reinterpret_cast<double2 *>(p);
+    const double2 a = q[0], b = q[1];
+    q[0] = make_double2(a.x + v[0], a.y + v[1]);
+    q[1] = make_double2(b.x + v[2], b.y + v[3]);
+}
+
+// What bounds both kernels: DRAM and L2 traffic of one pass over the adjoint
+// state, the forward images and the FP64 accumulators (about 220 bytes per
+// point in 2D with three mechanisms); so there is no tile with recomputed
+// halos: the adjoints of q_d and g_d go through global scratch (8 to 24 bytes
+// per point each way, mostly L2 hits from one kernel to the next).
+// Registers are held to four CTAs of 128 threads per SM in FP32.
+template <typename R, int DIM, int NM>
+__global__ void __launch_bounds__(32 * kAdjRows, sizeof(R) == 4 ? 4 : 1) k_adj_pressure(const __grid_constant__ AdjArgs<R> A)
+{
+    const AdjPos P = adj_pos<R, DIM>(A);
+    if (!P.on) return;
+    R lp[4], kd[4], q[3][4], div[4], d[4];
+    Io<R>::ld(A.L.lp + P.i, lp);
+    adj_diff<R, 0, false>(A, P, A.Gd[0], d);
 #pragma unroll
-        for (int ax = 0; ax < 3; ++ax)
-            if (DIM == 3 || ax != 1) {
-                q[ax] = dminus(A, A.fv1[ax], i, P.c[ax], P.n[ax], P.st[ax]);
-                div += q[ax];
-            }
+    for (int e = 0; e < 4; ++e) div[e] = d[e];
+    if (DIM == 3) {
+        adj_diff<R, 1, false>(A, P, A.Gd[1], d);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) div[e] += d[e];
     }
-    const R lp = __ldg(A.in.lp + i);
-    const R lst = -__ldg(A.kdt + i) * lp;
-    // tissue ramp of the absorbing layer: a -> r a (the forward sweep's ce, r div)
-    const R r = cell_ramp(A, P);
-    const R ce = __ldg(t + 3) + (r - R(1)) * __ldg(t + kLutDk + 1);   // the forward sweep's ceff
-    R stp = div * ce;
-    R ldiv = ce * lst;
-    // this step's terms in the working precision; the sum over steps in FP64
-    // (FP64 arithmetic is slow on this GPU: one addition per point and step)
-    gs = 0;
+    adj_diff<R, 2, false>(A, P, A.Gd[2], d);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) lp[e] = P.c[0] + e < A.nx ? lp[e] - (div[e] + d[e]) : R(0);
+    Io<R>::st(A.L.lp + P.i, lp);
+    adj_diff<R, 0, false>(A, P, A.fv1[0], q[0]);
+    adj_diff<R, 2, false>(A, P, A.fv1[2], q[2]);
+    if (DIM == 3) adj_diff<R, 1, false>(A, P, A.fv1[1], q[1]);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) div[e] = DIM == 3 ? q[0][e] + q[2][e] + q[1][e] : q[0][e] + q[2][e];
+    Io<R>::ldg(A.kdt + P.i, kd);
+    uint16_t cls[4];
+    quad_classes(__ldg(reinterpret_cast<const uint2 *>(A.cls + P.i)), cls);
+    R ln[NM][4], old[NM][4];
 #pragma unroll
     for (int m = 0; m < NM; ++m) {
-        const R ln = __ldg(A.in.lpsi2[m] + i);
-        ldiv += r * __ldg(t + kLutA2 + m) * ln;
-        if (FULL) {
-            const R old = __ldg(A.fpsi2[m] + i);
-            stp += __ldg(t + kLutH2 + m) * old;
-            gs += (__ldg(dtb + 12 + m) * old + r * __ldg(dtb + 8 + m) * div) * (ln + R(0.5) * lst);
-            A.out.lpsi2[m][i] = __ldg(t + kLutB2 + m) * ln + __ldg(t + kLutH2 + m) * lst;
-        }
+        Io<R>::ld(A.L.lpsi2[m] + P.i, ln[m]);
+        Io<R>::ld(A.fpsi2[m] + P.i, old[m]);
     }
+    const bool in[3] = {adj_in_layer<R, DIM>(A, P, 0), adj_in_layer<R, DIM>(A, P, 1), adj_in_layer<R, DIM>(A, P, 2)};
+    R Q[4], gsp[4], stp[4], lst[4];
+    CellCoef<R, NM> C;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        if (e == 0 || cls[e] != cls[e - 1]) C.load(A, cls[e], 2);
+        const R r = in[0] || in[1] || in[2] ? adj_ramp(A, P, e) : R(1);
+        lst[e] = -kd[e] * lp[e];
+        const R rdiv = r * div[e], half = R(0.5) * lst[e];
+        R lq = R(0), mem = R(0), gs = R(0);
+#pragma unroll
+        for (int m = 0; m < NM; ++m) {
+            const R t = ln[m][e] + half, o = old[m][e];
+            lq += C.a[m] * t;
+            mem += o + (C.b[m] * o + C.a[m] * rdiv);
+            gs += (C.db[m] * o + C.da[m] * rdiv) * t;
+            ln[m][e] = C.b[m] * t + half;
+        }
+        Q[e] = fma(C.ik, lst[e], fma(C.il, lst[e], r * lq));
+        stp[e] = fma(C.ik, div[e], fma(C.il, div[e], R(0.5) * mem));
+        gsp[e] = gs;
+    }
+#pragma unroll
+    for (int m = 0; m < NM; ++m) Io<R>::st(A.L.lpsi2[m] + P.i, ln[m]);
+    Io<R>::st(A.gsp + P.i, gsp);
 #pragma unroll
     for (int ax = 0; ax < 3; ++ax) {
         if (DIM == 2 && ax == 1) continue;
-        R qv = ldiv;
-        if (A.pdi[ax]) {
-            const R d = __ldg(A.pdi[ax] + P.c[ax]);
-            if (d > R(0)) {
-                R a, b;
-                pml_ab(d, __ldg(A.pai[ax] + P.c[ax]), __ldg(t + 1), A.dt, a, b);
-                const R ln = __ldg(A.in.lpsi2p[ax] + i);
-                qv += a * (ln + R(0.5) * lst);
-                if (FULL) {
-                    const R old = __ldg(A.fpsi2p[ax] + i);
-                    stp += R(0.5) * (R(1) + b) * old + R(0.5) * a * q[ax];
-                    A.out.lpsi2p[ax][i] = b * ln + R(0.5) * (R(1) + b) * lst;
-                }
+        R Qa[4] = {Q[0], Q[1], Q[2], Q[3]};
+        if (in[ax]) {
+            R a[4], b[4], lpn[4], po[4];
+            if (ax == 0) {
+                const R *pd = A.pdi[0] + P.c[0], *pa = A.pai[0] + P.c[0];
+                const R dq[4] = {pd[0], pd[1], pd[2], pd[3]}, aq[4] = {pa[0], pa[1], pa[2], pa[3]};
+                quad_layer_ab(A.lut, cls, 1, dq, aq, A.dt, a, b);
+            } else {
+                quad_layer_ab(A.lut, cls, 1, A.pdi[ax][P.c[ax]], A.pai[ax][P.c[ax]], A.dt, a, b);
             }
+            Io<R>::ld(A.L.lpsi2p[ax] + P.i, lpn);
+            Io<R>::ld(A.fpsi2p[ax] + P.i, po);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                if (!(b[e] <= R(1)) || P.c[0] + e >= A.nx) continue;   // zero profile, dead lane
+                Qa[e] += a[e] * (lpn[e] + R(0.5) * lst[e]);
+                stp[e] += R(0.5) * (R(1) + b[e]) * po[e] + R(0.5) * a[e] * q[ax][e];
+                lpn[e] = b[e] * lpn[e] + R(0.5) * (R(1) + b[e]) * lst[e];
+            }
+            Io<R>::st(A.L.lpsi2p[ax] + P.i, lpn);
         }
-        Qv[ax] = qv;
+        Io<R>::st(A.Q[ax] + P.i, Qa);
     }
-    gk = FULL ? double(-stp * lp) : 0.0;
+    double gk[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) gk[e] = double(-stp[e] * lp[e]);
+    add4(A.gk + P.i, gk);
 }
 
-// Velocity adjoint along axis ax at an in-grid point i, given dq = D+ of the
-// adjoint of q_ax there: returns the adjoint of g_ax.  FULL also adds the
-// gradient terms to gs and writes v_ax and the memory variables before the
-// step.
-template <typename R, int NM, bool FULL, int ax>
-__device__ __forceinline__ R vel_point(const AdjArgs<R> &A, const Pt<R> &P, long long i, R dq, R &gs)
+// velocity adjoint along ax; adds its terms to gs
+template <typename R, int DIM, int NM, int ax>
+__device__ __forceinline__ void adj_velocity_axis(const AdjArgs<R> &A, const AdjPos &P, const uint16_t (&cls)[4],
+                                                  const R (&own)[4], const R (&rr)[4], R (&gs)[4])
 {
-    const int cl = __ldg(A.cls + i);
-    const R *t = A.lut + (size_t)cl * kLutStride;
-    const R *dtb = A.dlut + (size_t)cl * kDStride;
-    const R own = __ldg(A.rho + i);
-    const R r = cell_ramp(A, P);
-    const R ce = __ldg(t + 2) + (r - R(1)) * __ldg(t + kLutDk);
-    const int c = P.c[ax], n = P.n[ax];
-    const long long st = P.st[ax];
-    const R lv = __ldg(A.in.lv[ax] + i) - dq;
-    const R nxt = (c + 1 < n) ? __ldg(A.rho + i + st) : own;
-    const R dtr = R(2) * A.dt * fw_rcp(own + nxt);
-    const R lst = -dtr * lv;
-    const R g = FULL ? dplus(A, A.fp, i, c, n, st) : R(0);
-    R lg = ce * lst;
+    R lv[4], dq[4], g[4], nxt[4], ln[NM][4], old[NM][4], lg[4], lst[4];
+    Io<R>::ld(A.L.lv[ax] + P.i, lv);
 #pragma unroll
     for (int m = 0; m < NM; ++m) {
-        const R ln = __ldg(A.in.lpsi1[m][ax] + i);
-        lg += r * __ldg(t + kLutA1 + m) * ln;
-        if (FULL) {
-            const R old = __ldg(A.fpsi1[m][ax] + i);
-            gs += (__ldg(dtb + 4 + m) * old + r * __ldg(dtb + m) * g) * (ln + R(0.5) * lst);
-            A.out.lpsi1[m][ax][i] = __ldg(t + kLutB1 + m) * ln + __ldg(t + kLutH1 + m) * lst;
+        Io<R>::ld(A.L.lpsi1[m][ax] + P.i, ln[m]);
+        Io<R>::ld(A.fpsi1[m][ax] + P.i, old[m]);
+    }
+    adj_diff<R, ax, true>(A, P, A.Q[ax], dq);
+    adj_diff<R, ax, true>(A, P, A.fp, g);
+    if (ax == 0) {
+        nxt[0] = own[1]; nxt[1] = own[2]; nxt[2] = own[3];
+        nxt[3] = P.c[0] + 4 < A.nx ? __ldg(A.rho + P.i + 4) : own[3];
+    } else {
+        ld4_or_zero(A.rho + P.i + P.st[ax], P.c[ax] + 1 < P.n[ax], nxt);
+    }
+    CellCoef<R, NM> C;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const bool live = P.c[0] + e < A.nx;
+        if (ax == 0 ? P.c[0] + e + 1 >= A.nx : P.c[ax] + 1 >= P.n[ax]) nxt[e] = own[e];
+        if (e == 0 || cls[e] != cls[e - 1]) C.load(A, cls[e], 1);
+        lv[e] = live ? lv[e] - dq[e] : R(0);
+        lst[e] = live ? div_face(-A.dt, fma(R(0.5), nxt[e], R(0.5) * own[e])) * lv[e] : R(0);
+        const R rg = live ? rr[e] * g[e] : R(0), half = R(0.5) * lst[e];
+        R lq = R(0);
+#pragma unroll
+        for (int m = 0; m < NM; ++m) {
+            const R t = ln[m][e] + half, o = old[m][e];
+            lq += C.a[m] * t;
+            gs[e] += (C.db[m] * o + C.da[m] * rg) * t;
+            ln[m][e] = C.b[m] * t + half;
         }
+        lg[e] = fma(C.ik, lst[e], fma(C.il, lst[e], rr[e] * lq));
     }
-    if (A.pdh[ax]) {
-        const R d = __ldg(A.pdh[ax] + c);
-        if (d > R(0)) {
-            R a, b;
-            pml_ab(d, __ldg(A.pah[ax] + c), __ldg(t), A.dt, a, b);
-            const R ln = __ldg(A.in.lpsi1p[ax] + i);
-            lg += a * (ln + R(0.5) * lst);
-            if (FULL) A.out.lpsi1p[ax][i] = b * ln + R(0.5) * (R(1) + b) * lst;
+    Io<R>::st(A.L.lv[ax] + P.i, lv);
+#pragma unroll
+    for (int m = 0; m < NM; ++m) Io<R>::st(A.L.lpsi1[m][ax] + P.i, ln[m]);
+    if (adj_in_layer<R, DIM>(A, P, ax)) {
+        R a[4], b[4], lpn[4];
+        if (ax == 0) {
+            const R *pd = A.pdh[0] + P.c[0], *pa = A.pah[0] + P.c[0];
+            const R d4[4] = {pd[0], pd[1], pd[2], pd[3]}, a4[4] = {pa[0], pa[1], pa[2], pa[3]};
+            quad_layer_ab(A.lut, cls, 0, d4, a4, A.dt, a, b);
+        } else {
+            quad_layer_ab(A.lut, cls, 0, A.pdh[ax][P.c[ax]], A.pah[ax][P.c[ax]], A.dt, a, b);
         }
+        Io<R>::ld(A.L.lpsi1p[ax] + P.i, lpn);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            if (!(b[e] <= R(1)) || P.c[0] + e >= A.nx) continue;
+            lg[e] += a[e] * (lpn[e] + R(0.5) * lst[e]);
+            lpn[e] = b[e] * lpn[e] + R(0.5) * (R(1) + b[e]) * lst[e];
+        }
+        Io<R>::st(A.L.lpsi1p[ax] + P.i, lpn);
     }
-    if (FULL) A.out.lv[ax][i] = lv;
-    return lg;
-}
-
-// ---- three-kernel form (3D): adjoints of q_d and g_d through global scratch ----
-
-template <typename R, int DIM, int NM>
-__global__ void k_adj_pres(const AdjArgs<R> A)
-{
-    Pt<R> P;
-    long long i;
-    if (!point(A, P, i)) return;
-    R Qv[3], gs;
-    double gk;
-    pres_point<R, DIM, NM, true>(A, P, i, Qv, gs, gk);
-#pragma unroll
-    for (int ax = 0; ax < 3; ++ax)
-        if (DIM == 3 || ax != 1) A.Q[ax][i] = Qv[ax];
-    A.gk[i] += gk;
-    A.gs[i] += double(gs);
+    Io<R>::st(A.Gd[ax] + P.i, lg);
 }
 
 template <typename R, int DIM, int NM>
-__global__ void k_adj_vel(const AdjArgs<R> A)
+__global__ void __launch_bounds__(32 * kAdjRows, sizeof(R) == 4 ? 4 : 1) k_adj_velocity(const __grid_constant__ AdjArgs<R> A)
 {
-    Pt<R> P;
-    long long i;
-    if (!point(A, P, i)) return;
-    R gs = 0;   // this step's terms; the sum over steps in FP64
+    const AdjPos P = adj_pos<R, DIM>(A);
+    if (!P.on) return;
+    uint16_t cls[4];
+    quad_classes(__ldg(reinterpret_cast<const uint2 *>(A.cls + P.i)), cls);
+    R own[4], gs[4], rr[4] = {R(1), R(1), R(1), R(1)};
+    Io<R>::ldg(A.rho + P.i, own);
+    Io<R>::ld(A.gsp + P.i, gs);
+    if (adj_in_layer<R, DIM>(A, P, 0) || adj_in_layer<R, DIM>(A, P, 1) || adj_in_layer<R, DIM>(A, P, 2))
 #pragma unroll
-    for (int ax = 0; ax < 3; ++ax) {
-        if (DIM == 2 && ax == 1) continue;
-        const R dq = dplus(A, A.Q[ax], i, P.c[ax], P.n[ax], P.st[ax]);
-        A.Gd[ax][i] = ax == 0   ? vel_point<R, NM, true, 0>(A, P, i, dq, gs)
-                      : ax == 1 ? vel_point<R, NM, true, 1>(A, P, i, dq, gs)
-                                : vel_point<R, NM, true, 2>(A, P, i, dq, gs);
-    }
-    A.gs[i] += double(gs);
+        for (int e = 0; e < 4; ++e) rr[e] = adj_ramp(A, P, e);
+    adj_velocity_axis<R, DIM, NM, 0>(A, P, cls, own, rr, gs);
+    if (DIM == 3) adj_velocity_axis<R, DIM, NM, 1>(A, P, cls, own, rr, gs);
+    adj_velocity_axis<R, DIM, NM, 2>(A, P, cls, own, rr, gs);
+    const double g[4] = {double(gs[0]), double(gs[1]), double(gs[2]), double(gs[3])};
+    add4(A.gs + P.i, g);
 }
 
-template <typename R, int DIM, int NM>
-__global__ void k_adj_p(const AdjArgs<R> A)
-{
-    Pt<R> P;
-    long long i;
-    if (!point(A, P, i)) return;
-    R s = 0;
-#pragma unroll
-    for (int ax = 0; ax < 3; ++ax)
-        if (DIM == 3 || ax != 1) s += dminus(A, A.Gd[ax], i, P.c[ax], P.n[ax], P.st[ax]);
-    A.out.lp[i] = A.in.lp[i] - s;
-}
-
-// Transpose of the step's injection and recording (k_io), in one launch:
-// threads [0, n_src) add the adjoint of the receiver on the source's cell
-// (if any and if col >= 0) to the pressure adjoint there and take the
-// source-gain gradient of step it (it < wave_len) from it; threads
-// [n_src, n_src + n_rcv) add the adjoints of the other receivers (col >= 0).
+// Transpose of injection and recording (k_io), in one launch after the
+// pressure adjoint of step it: threads [0, n_src) take the source-gain
+// gradient of step it (it < wave_len; it < 0: none) from the pressure adjoint
+// at the source's cell, then add the adjoint of the earlier step's receiver on
+// that cell (col >= 0: its trace column); threads [n_src, n_src + n_rcv) add
+// those of the other receivers.
 template <typename R>
 __global__ void k_adj_io(R *lp, const long long *src_idx, const R *waves, const int *wave_of, int wave_len, int it,
                          int n_src, const int *src_rcv, const long long *rcv_idx, const int *rcv_src, const R *G,
@@ -323,12 +365,9 @@ __global__ void k_adj_io(R *lp, const long long *src_idx, const R *waves, const 
     if (t < n_src) {
         const long long k = src_idx[t];
         const int r = col >= 0 ? src_rcv[t] : -1;
-        R l = lp[k];
-        if (r >= 0) {
-            l += G[(size_t)r * n_col + col];
-            lp[k] = l;
-        }
-        if (it < wave_len) gk[k] += double(waves[(size_t)wave_of[t] * wave_len + it]) * double(l) * inv_dxd;
+        const R l = lp[k];
+        if (it >= 0 && it < wave_len) gk[k] += double(waves[(size_t)wave_of[t] * wave_len + it]) * double(l) * inv_dxd;
+        if (r >= 0) lp[k] = l + G[(size_t)r * n_col + col];
     } else if (col >= 0 && t < n_src + n_rcv) {
         const int r = t - n_src;
         if (rcv_src[r] >= 0) return;     // added by the thread of the source on its cell
@@ -380,422 +419,28 @@ __global__ void k_grad_out(const double *uc, const double *us, const float *a0f,
     }
 }
 
-// ---- one-kernel form (2D): the whole reverse step per tile ----
-//
-// A CTA owns a TX x TZ tile of the (x, z) grid.  The adjoints of q_d and g_d
-// stay in shared memory over the tile and the halo their two stencils need
-// along their own axis: g_d on 4 points before and 3 after the tile (the
-// backward difference of the last update), q_d on 7 before and 7 after (the
-// forward difference that gives g_d there).  Each CTA recomputes its halo from
-// the adjoint state after the step, which it reads from one buffer while it
-// writes the state before the step to the other (a neighbour still reads the
-// old values).
-// tuning overrides: FWGB_ADJ_TX / FWGB_ADJ_TZ (tile), FWGB_ADJ_THREADS
-#ifndef FWGB_ADJ_THREADS
-#define FWGB_ADJ_THREADS 256
-#endif
-#ifndef FWGB_ADJ_TX
-#define FWGB_ADJ_TX 32
-#endif
-#ifndef FWGB_ADJ_TZ
-#define FWGB_ADJ_TZ 32
-#endif
-constexpr int kAdjThreads = FWGB_ADJ_THREADS;
-
-template <int TX, int TZ> struct AdjTile {
-    static constexpr int QXW = TX + 14, QZH = TZ + 14;   // q_x rows, q_z columns
-    static constexpr int GXW = TX + 7, GZH = TZ + 7;     // g_x rows, g_z columns
-    static constexpr int FPW = TX + 7, FPH = TZ + 7;     // forward p: columns x0-3 .., rows z0-3 ..
-    static constexpr int n_qx = TZ * QXW, n_qz = QZH * TX, n_gx = TZ * GXW, n_gz = GZH * TX;
-    static constexpr int n_fp = FPH * FPW, n_v0 = TZ * (TX + 7), n_v2 = (TZ + 7) * TX;
-    static constexpr int elems = n_qx + n_qz + n_gx + n_gz + n_fp + n_v0 + n_v2;
-    static constexpr int NI = TX * TZ / kAdjThreads;     // tile points per thread
-    static_assert(TX * TZ % kAdjThreads == 0, "tile points split evenly over the threads");
-};
-
-// ---- one-kernel form (2D) ----
-// tissue-mechanism strength of the cell (x, z) (cell_ramp of a 2D grid)
-template <typename R>
-__device__ __forceinline__ R ramp2(const AdjArgs<R> &A, int x, int z)
+template <typename R, int DIM, int NM>
+cudaError_t launch_reverse_n(const AdjArgs<R> &A, int side, cudaStream_t s)
 {
-    const R s = fmax(layer_depth<R>(x, A.nx, A.wabs), layer_depth<R>(z, A.nz, A.wabs));
-    return ramp_of(s, A.inv_lr);
-}
-
-// Pressure adjoint at an in-grid point i = (x, z) of class table t / dtb and
-// tissue strength r: the adjoints of q_x and q_z (Qx, Qz; the halo needs one
-// of them, ONLY = 0 or 2).  FULL: qx, qz are the forward D- differences of
-// v after the step at the point; takes this step's gradient terms (gs, gk)
-// and writes the memory variables before the step.  PLAIN: no absorbing
-// layer within reach of the tile (r = 1, no layer memory).
-template <typename R, int NM, bool FULL, bool PLAIN, int ONLY = -1>
-__device__ __forceinline__ void pres2(const AdjArgs<R> &A, int x, int z, long long i, const R *t, const R *dtb, R r,
-                                      R qx, R qz, R &Qx, R &Qz, R &gs, double &gk)
-{
-    const R div = qx + qz;
-    const R lp = __ldg(A.in.lp + i);
-    const R lst = -__ldg(A.kdt + i) * lp;
-    const R ce = PLAIN ? __ldg(t + 3) : __ldg(t + 3) + (r - R(1)) * __ldg(t + kLutDk + 1);
-    R stp = div * ce;
-    R ldiv = ce * lst;
-    gs = 0;
-#pragma unroll
-    for (int m = 0; m < NM; ++m) {
-        const R ln = __ldg(A.in.lpsi2[m] + i);
-        ldiv += (PLAIN ? R(1) : r) * __ldg(t + kLutA2 + m) * ln;
-        if (FULL) {
-            const R old = __ldg(A.fpsi2[m] + i);
-            const R h = __ldg(t + kLutH2 + m);
-            stp += h * old;
-            gs += (__ldg(dtb + 12 + m) * old + (PLAIN ? R(1) : r) * __ldg(dtb + 8 + m) * div) * (ln + R(0.5) * lst);
-            A.out.lpsi2[m][i] = __ldg(t + kLutB2 + m) * ln + h * lst;
-        }
-    }
-    Qx = Qz = ldiv;
-    if (!PLAIN) {
-#pragma unroll
-        for (int ax = 0; ax < 3; ax += 2) {
-            if (ONLY >= 0 && ax != ONLY) continue;
-            if (!A.pdi[ax]) continue;
-            const int c = ax == 0 ? x : z;
-            const R d = __ldg(A.pdi[ax] + c);
-            if (d > R(0)) {
-                R a, b;
-                pml_ab(d, __ldg(A.pai[ax] + c), __ldg(t + 1), A.dt, a, b);
-                const R ln = __ldg(A.in.lpsi2p[ax] + i);
-                (ax == 0 ? Qx : Qz) += a * (ln + R(0.5) * lst);
-                if (FULL) {
-                    const R old = __ldg(A.fpsi2p[ax] + i);
-                    stp += R(0.5) * (R(1) + b) * old + R(0.5) * a * (ax == 0 ? qx : qz);
-                    A.out.lpsi2p[ax][i] = b * ln + R(0.5) * (R(1) + b) * lst;
-                }
-            }
-        }
-    }
-    gk = FULL ? double(-stp * lp) : 0.0;
-}
-
-// Velocity adjoint along axis ax (0 or 2) at an in-grid point i, coordinate c
-// of n along ax, stride st: given dq = D+ of the adjoint of q_ax there,
-// returns the adjoint of g_ax.  FULL: g is the forward D+ difference of p
-// before the step; adds the gradient terms to gs and writes v_ax and the
-// memory variables before the step.
-template <typename R, int NM, bool FULL, bool PLAIN, int ax>
-__device__ __forceinline__ R vel2(const AdjArgs<R> &A, int c, int n, long long st, long long i, const R *t,
-                                  const R *dtb, R r, R dq, R g, R &gs)
-{
-    const R own = __ldg(A.rho + i);
-    const R ce = PLAIN ? __ldg(t + 2) : __ldg(t + 2) + (r - R(1)) * __ldg(t + kLutDk);
-    const R lv = __ldg(A.in.lv[ax] + i) - dq;
-    const R nxt = (c + 1 < n) ? __ldg(A.rho + i + st) : own;
-    const R dtr = R(2) * A.dt * fw_rcp(own + nxt);
-    const R lst = -dtr * lv;
-    R lg = ce * lst;
-#pragma unroll
-    for (int m = 0; m < NM; ++m) {
-        const R ln = __ldg(A.in.lpsi1[m][ax] + i);
-        lg += (PLAIN ? R(1) : r) * __ldg(t + kLutA1 + m) * ln;
-        if (FULL) {
-            const R old = __ldg(A.fpsi1[m][ax] + i);
-            gs += (__ldg(dtb + 4 + m) * old + (PLAIN ? R(1) : r) * __ldg(dtb + m) * g) * (ln + R(0.5) * lst);
-            A.out.lpsi1[m][ax][i] = __ldg(t + kLutB1 + m) * ln + __ldg(t + kLutH1 + m) * lst;
-        }
-    }
-    if (!PLAIN && A.pdh[ax]) {
-        const R d = __ldg(A.pdh[ax] + c);
-        if (d > R(0)) {
-            R a, b;
-            pml_ab(d, __ldg(A.pah[ax] + c), __ldg(t), A.dt, a, b);
-            const R ln = __ldg(A.in.lpsi1p[ax] + i);
-            lg += a * (ln + R(0.5) * lst);
-            if (FULL) A.out.lpsi1p[ax][i] = b * ln + R(0.5) * (R(1) + b) * lst;
-        }
-    }
-    if (FULL) A.out.lv[ax][i] = lv;
-    return lg;
-}
-
-#ifndef FWGB_ADJ_PREFETCH
-#define FWGB_ADJ_PREFETCH 2   // 0: none, 1: both sides at the start, 2: velocity side after the tile's q_d
-#endif
-
-// Bulk prefetch into L2 of the elements [xa, xb) of row z of a field, clamped
-// to the row (rows are 128-byte aligned, so the 16-byte rounding stays inside).
-template <typename R, typename T>
-__device__ __forceinline__ void prefetch_row(const AdjArgs<R> &A, const T *f, int z, int xa, int xb)
-{
-    xa = max(xa, 0);
-    xb = min(xb, A.px);
-    if (!f || z < 0 || z >= A.nz || xa >= xb) return;
-    const size_t b = __cvta_generic_to_global(f + (long long)z * A.plane + xa) & ~size_t(15);
-    const size_t e = (__cvta_generic_to_global(f + (long long)z * A.plane + xb) + 15) & ~size_t(15);
-    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(b), "r"((unsigned)(e - b)) : "memory");
-}
-
-// The fields one side of the reverse step reads on a tile (side 0: pressure
-// adjoint, side 1: velocity adjoint), field f of that side: its pointer and
-// whether it is read on the q_d halo box (else on the tile with a 4-point
-// stencil halo).
-template <typename R, int NM>
-__device__ __forceinline__ int side_fields(int side) { return side == 0 ? 6 + 2 * NM : 5 + 4 * NM; }
-
-template <typename R, int NM>
-__device__ __forceinline__ void side_field(const AdjArgs<R> &A, int side, int f, const void *&p, int &es, bool &box)
-{
-    es = sizeof(R);
-    box = true;
-    if (side == 0) {
-        if (f == 0) p = A.in.lp;
-        else if (f == 1) p = A.kdt;
-        else if (f == 2) { p = A.cls; es = 2; }
-        else if (f < 3 + NM) p = A.in.lpsi2[f - 3];
-        else {
-            box = false;
-            f -= 3 + NM;
-            if (f == 0) p = A.fv1[0];
-            else if (f == 1) p = A.fv1[2];
-            else if (f == 2) { p = A.gk; es = 8; }
-            else p = A.fpsi2[f - 3];
-        }
-    } else {
-        if (f == 0) p = A.in.lv[0];
-        else if (f == 1) p = A.in.lv[2];
-        else if (f == 2) p = A.rho;
-        else if (f < 3 + NM) p = A.in.lpsi1[f - 3][0];
-        else if (f < 3 + 2 * NM) p = A.in.lpsi1[f - 3 - NM][2];
-        else {
-            box = false;
-            f -= 3 + 2 * NM;
-            if (f == 0) p = A.fp;
-            else if (f == 1) { p = A.gs; es = 8; }
-            else if (f < 2 + NM) p = A.fpsi1[f - 2][0];
-            else p = A.fpsi1[f - 2 - NM][2];
-        }
-    }
-}
-
-template <typename R, int NM, int TX, int TZ>
-__device__ __forceinline__ void prefetch_side(const AdjArgs<R> &A, int side, int x0, int z0)
-{
-    constexpr int ROWS = TZ + 14;
-    const int n = side_fields<R, NM>(side) * ROWS;
-    for (int j = threadIdx.x; j < n; j += kAdjThreads) {
-        const int f = j / ROWS, r = j % ROWS;
-        const void *p;
-        int es;
-        bool box;
-        side_field<R, NM>(A, side, f, p, es, box);
-        const int h = box ? 7 : 4;
-        if (r >= TZ + 2 * h) continue;
-        const int z = z0 - h + r, xa = x0 - h, xb = x0 + TX + h;
-        if (es == 2) prefetch_row(A, static_cast<const uint16_t *>(p), z, xa, xb);
-        else if (es == 4) prefetch_row(A, static_cast<const float *>(p), z, xa, xb);
-        else prefetch_row(A, static_cast<const double *>(p), z, xa, xb);
-    }
-}
-
-// The reverse step on one TX x TZ tile: the pressure adjoint on the tile and
-// on the q_d halo (7 points either side along d), the velocity adjoint on the
-// tile and on the g_d halo (4 before, 3 after), then the update of the
-// pressure adjoint on the tile.  The forward fields whose differences the
-// step takes (p before the step, v after it) are staged in shared memory
-// with their halos, zero beyond the grid.
-template <typename R, int NM, int TX, int TZ, bool PLAIN>
-__device__ __forceinline__ void step2_tile(const AdjArgs<R> &A, unsigned char *smem, int x0, int z0)
-{
-    using T = AdjTile<TX, TZ>;
-    R *sQx = reinterpret_cast<R *>(smem);
-    R *sQz = sQx + T::n_qx;
-    R *sGx = sQz + T::n_qz;
-    R *sGz = sGx + T::n_gx;
-    R *sFP = sGz + T::n_gz;   // p before the step: rows z0-3 .. z0+TZ+3, columns x0-3 .. x0+TX+3
-    R *sV0 = sFP + T::n_fp;   // v_x after it: rows z0 .. z0+TZ-1, columns x0-4 .. x0+TX+2
-    R *sV2 = sV0 + T::n_v0;   // v_z after it: rows z0-4 .. z0+TZ+2, columns x0 .. x0+TX-1
-    const int tid = threadIdx.x;
-    auto inside = [&](int x, int z) { return x >= 0 && x < A.nx && z >= 0 && z < A.nz; };
-    auto at = [&](int x, int z) { return (long long)z * A.plane + x; };
-    auto tab = [&](int cl) { return A.lut + (size_t)cl * kLutStride; };
-    auto dtab = [&](int cl) { return A.dlut + (size_t)cl * kDStride; };
-
-    for (int j = tid; j < T::n_fp; j += kAdjThreads) {
-        const int x = x0 - 3 + j % T::FPW, z = z0 - 3 + j / T::FPW;
-        sFP[j] = inside(x, z) ? __ldg(A.fp + at(x, z)) : R(0);
-    }
-    for (int j = tid; j < T::n_v0; j += kAdjThreads) {
-        const int x = x0 - 4 + j % (TX + 7), z = z0 + j / (TX + 7);
-        sV0[j] = inside(x, z) ? __ldg(A.fv1[0] + at(x, z)) : R(0);
-    }
-    for (int j = tid; j < T::n_v2; j += kAdjThreads) {
-        const int x = x0 + j % TX, z = z0 - 4 + j / TX;
-        sV2[j] = inside(x, z) ? __ldg(A.fv1[2] + at(x, z)) : R(0);
-    }
-    __syncthreads();
-
-    R gsum[T::NI], rk[T::NI];
-    int clk[T::NI];
-    // q_d: the tile (full pressure adjoint), then the wings
-#pragma unroll
-    for (int k = 0; k < T::NI; ++k) {
-        const int j = tid + k * kAdjThreads, lx = j % TX, lz = j / TX, x = x0 + lx, z = z0 + lz;
-        R Qx = 0, Qz = 0;
-        gsum[k] = 0;
-        clk[k] = 0;
-        rk[k] = R(1);
-        if (inside(x, z)) {
-            const long long i = at(x, z);
-            const int cl = __ldg(A.cls + i);
-            const R r = PLAIN ? R(1) : ramp2(A, x, z);
-            clk[k] = cl;
-            rk[k] = r;
-            const R qx = dminus_s(A, &sV0[lz * (TX + 7) + lx + 4], 1);
-            const R qz = dminus_s(A, &sV2[(lz + 4) * TX + lx], TX);
-            double gk;
-            pres2<R, NM, true, PLAIN>(A, x, z, i, tab(cl), dtab(cl), r, qx, qz, Qx, Qz, gsum[k], gk);
-            A.gk[i] += gk;
-        }
-        sQx[lz * T::QXW + lx + 7] = Qx;
-        sQz[(lz + 7) * TX + lx] = Qz;
-    }
-    if (FWGB_ADJ_PREFETCH == 2) prefetch_side<R, NM, TX, TZ>(A, 1, x0, z0);
-    for (int j = tid; j < 14 * (TZ + TX); j += kAdjThreads) {
-        int lx, lz;
-        const bool along_x = j < 14 * TZ;
-        if (along_x) {       // q_x: 7 points either side of each tile row
-            const int w = j % 14;
-            lz = j / 14;
-            lx = w < 7 ? w - 7 : TX + w - 7;
-        } else {             // q_z: 7 rows above and below the tile
-            const int jj = j - 14 * TZ, w = jj / TX;
-            lx = jj % TX;
-            lz = w < 7 ? w - 7 : TZ + w - 7;
-        }
-        const int x = x0 + lx, z = z0 + lz;
-        R Qx = 0, Qz = 0;
-        if (inside(x, z)) {
-            const long long i = at(x, z);
-            const int cl = __ldg(A.cls + i);
-            const R r = PLAIN ? R(1) : ramp2(A, x, z);
-            R gs;
-            double gk;
-            if (along_x) pres2<R, NM, false, PLAIN, 0>(A, x, z, i, tab(cl), dtab(cl), r, R(0), R(0), Qx, Qz, gs, gk);
-            else pres2<R, NM, false, PLAIN, 2>(A, x, z, i, tab(cl), dtab(cl), r, R(0), R(0), Qx, Qz, gs, gk);
-        }
-        if (along_x) sQx[lz * T::QXW + lx + 7] = Qx;
-        else sQz[(lz + 7) * TX + lx] = Qz;
-    }
-    __syncthreads();
-
-    // g_d: the tile (full velocity adjoint along both axes), then the wings
-#pragma unroll
-    for (int k = 0; k < T::NI; ++k) {
-        const int j = tid + k * kAdjThreads, lx = j % TX, lz = j / TX, x = x0 + lx, z = z0 + lz;
-        R gx = 0, gz = 0;
-        if (inside(x, z)) {
-            const long long i = at(x, z);
-            const R *t = tab(clk[k]), *dtb = dtab(clk[k]);
-            const R *fp = &sFP[(lz + 3) * T::FPW + lx + 3];
-            gx = vel2<R, NM, true, PLAIN, 0>(A, x, A.nx, 1, i, t, dtb, rk[k], dplus_s(A, &sQx[lz * T::QXW + lx + 7], 1),
-                                             dplus_s(A, fp, 1), gsum[k]);
-            gz = vel2<R, NM, true, PLAIN, 2>(A, z, A.nz, A.plane, i, t, dtb, rk[k],
-                                             dplus_s(A, &sQz[(lz + 7) * TX + lx], TX), dplus_s(A, fp, T::FPW), gsum[k]);
-        }
-        sGx[lz * T::GXW + lx + 4] = gx;
-        sGz[(lz + 4) * TX + lx] = gz;
-    }
-    for (int j = tid; j < 7 * (TZ + TX); j += kAdjThreads) {
-        int lx, lz;
-        const bool along_x = j < 7 * TZ;
-        if (along_x) {       // g_x: 4 points before and 3 after each tile row
-            const int w = j % 7;
-            lz = j / 7;
-            lx = w < 4 ? w - 4 : TX + w - 4;
-        } else {             // g_z: 4 rows above and 3 below the tile
-            const int jj = j - 7 * TZ, w = jj / TX;
-            lx = jj % TX;
-            lz = w < 4 ? w - 4 : TZ + w - 4;
-        }
-        const int x = x0 + lx, z = z0 + lz;
-        R g = 0, unused = 0;
-        if (inside(x, z)) {
-            const long long i = at(x, z);
-            const int cl = __ldg(A.cls + i);
-            const R r = PLAIN ? R(1) : ramp2(A, x, z);
-            g = along_x ? vel2<R, NM, false, PLAIN, 0>(A, x, A.nx, 1, i, tab(cl), dtab(cl), r,
-                                                       dplus_s(A, &sQx[lz * T::QXW + lx + 7], 1), R(0), unused)
-                        : vel2<R, NM, false, PLAIN, 2>(A, z, A.nz, A.plane, i, tab(cl), dtab(cl), r,
-                                                       dplus_s(A, &sQz[(lz + 7) * TX + lx], TX), R(0), unused);
-        }
-        if (along_x) sGx[lz * T::GXW + lx + 4] = g;
-        else sGz[(lz + 4) * TX + lx] = g;
-    }
-    __syncthreads();
-
-    // p: the backward differences of g_d on the tile
-#pragma unroll
-    for (int k = 0; k < T::NI; ++k) {
-        const int j = tid + k * kAdjThreads, lx = j % TX, lz = j / TX, x = x0 + lx, z = z0 + lz;
-        if (!inside(x, z)) continue;
-        const R s = dminus_s(A, &sGx[lz * T::GXW + lx + 4], 1) + dminus_s(A, &sGz[(lz + 4) * TX + lx], TX);
-        const long long i = at(x, z);
-        A.out.lp[i] = __ldg(A.in.lp + i) - s;
-        A.gs[i] += double(gsum[k]);
-    }
-}
-
-// Tiles whose reads (the q_d halo reaches 7 cells, one more for the velocity
-// adjoint's neighbouring density) stay clear of the absorbing layer take the
-// PLAIN instance: no layer memory, tissue strength 1.  Registers are held
-// to four CTAs per SM (64 per thread) in FP32, two in FP64.
-template <typename R, int NM, int TX, int TZ>
-__global__ void __launch_bounds__(kAdjThreads, sizeof(R) == 4 ? 4 : 2) k_adj_step2(const AdjArgs<R> A)
-{
-    extern __shared__ __align__(16) unsigned char adj_smem[];
-    const int x0 = blockIdx.x * TX, z0 = blockIdx.y * TZ;
-    if (FWGB_ADJ_PREFETCH >= 1) prefetch_side<R, NM, TX, TZ>(A, 0, x0, z0);
-    if (FWGB_ADJ_PREFETCH == 1) prefetch_side<R, NM, TX, TZ>(A, 1, x0, z0);
-    constexpr int h = 8;
-    const bool plain = A.wabs <= 0 || (x0 - h >= A.wabs && x0 + TX + h <= A.nx - A.wabs && z0 - h >= A.wabs &&
-                                       z0 + TZ + h <= A.nz - A.wabs);
-    if (plain) step2_tile<R, NM, TX, TZ, true>(A, adj_smem, x0, z0);
-    else step2_tile<R, NM, TX, TZ, false>(A, adj_smem, x0, z0);
-}
-
-constexpr int kAdjTX = FWGB_ADJ_TX, kAdjTZ = FWGB_ADJ_TZ;
-
-template <typename R, int NM>
-cudaError_t launch_step2_n(const AdjArgs<R> &A, cudaStream_t s, bool setup)
-{
-    using T = AdjTile<kAdjTX, kAdjTZ>;
-    const size_t smem = (size_t)T::elems * sizeof(R);
-    if (setup) return cudaFuncSetAttribute(k_adj_step2<R, NM, kAdjTX, kAdjTZ>,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    const dim3 grid((unsigned)((A.nx + kAdjTX - 1) / kAdjTX), (unsigned)((A.nz + kAdjTZ - 1) / kAdjTZ));
-    k_adj_step2<R, NM, kAdjTX, kAdjTZ><<<grid, kAdjThreads, smem, s>>>(A);
+    const unsigned gx = (unsigned)(A.nx + 127) / 128;
+    const unsigned rows = DIM == 3 ? (unsigned)(A.ny + kAdjRows - 1) / kAdjRows * (unsigned)A.nz
+                                   : (unsigned)(A.nz + kAdjRows - 1) / kAdjRows;
+    if (side == 2) k_adj_pressure<R, DIM, NM><<<gx * rows, dim3(32, kAdjRows), 0, s>>>(A);
+    else k_adj_velocity<R, DIM, NM><<<gx * rows, dim3(32, kAdjRows), 0, s>>>(A);
     return cudaGetLastError();
 }
 
-// the reverse step's kernels: one in 2D, three in 3D; instantiated per
-// dimension and number of mechanisms (their loops unroll).  With setup, only
-// the one-kernel form's shared-memory opt-in.
-template <typename R, int NM>
-cudaError_t launch_reverse_n(const AdjArgs<R> &A, int ndim, dim3 grid, cudaStream_t s, bool setup)
-{
-    if (ndim == 2) return launch_step2_n<R, NM>(A, s, setup);
-    if (setup) return cudaSuccess;
-    k_adj_pres<R, 3, NM><<<grid, 256, 0, s>>>(A);
-    k_adj_vel<R, 3, NM><<<grid, 256, 0, s>>>(A);
-    k_adj_p<R, 3, NM><<<grid, 256, 0, s>>>(A);
-    return cudaGetLastError();
-}
-
+// one half of a reverse step (side 2: pressure, 1: velocity); instances per
+// dimension and number of mechanisms (their loops unroll)
 template <typename R>
-cudaError_t launch_reverse(const AdjArgs<R> &A, int ndim, int nmech, dim3 grid, cudaStream_t s, bool setup = false)
+cudaError_t launch_reverse(const AdjArgs<R> &A, int ndim, int nmech, int side, cudaStream_t s)
 {
+    const bool d3 = ndim == 3;
     switch (nmech) {
-    case 1: return launch_reverse_n<R, 1>(A, ndim, grid, s, setup);
-    case 2: return launch_reverse_n<R, 2>(A, ndim, grid, s, setup);
-    case 3: return launch_reverse_n<R, 3>(A, ndim, grid, s, setup);
-    default: return launch_reverse_n<R, 4>(A, ndim, grid, s, setup);
+    case 1: return d3 ? launch_reverse_n<R, 3, 1>(A, side, s) : launch_reverse_n<R, 2, 1>(A, side, s);
+    case 2: return d3 ? launch_reverse_n<R, 3, 2>(A, side, s) : launch_reverse_n<R, 2, 2>(A, side, s);
+    case 3: return d3 ? launch_reverse_n<R, 3, 3>(A, side, s) : launch_reverse_n<R, 2, 3>(A, side, s);
+    default: return d3 ? launch_reverse_n<R, 3, 4>(A, side, s) : launch_reverse_n<R, 2, 4>(A, side, s);
     }
 }
 
@@ -858,26 +503,22 @@ int gradient_impl(fw_medium *m, int n_steps, int K, const void *G, const void *a
     char *slab = static_cast<char *>(m->slab);
     auto off = [slab](const void *p) { return (size_t)(static_cast<const char *>(p) - slab); };
 
-    // 2D: one kernel per reverse step, reading the adjoint state from one of a
-    // pair of buffers and writing the other; 3D: three kernels in place, with
-    // the adjoints of q_d and g_d in global scratch.
-    const bool one_kernel = m->ndim == 2;
     // segment images: the states after steps k0 .. k1-2 of a segment (the state
     // before it is its checkpoint, the state after it the next checkpoint)
-    Buf lam(SB), lam2(one_kernel ? SB : 0), ck((size_t)n_ck * SB), fin(SB);
+    Buf lam(SB), ck((size_t)n_ck * SB), fin(SB);
     Buf seg0((size_t)std::max(seg_len - 1, 1) * SB), seg1(n_ck > 1 ? (size_t)std::max(seg_len - 1, 1) * SB : 0);
-    Buf scratch(one_kernel ? 0 : 6 * vol * sizeof(R)), gacc(2 * vol * sizeof(double)),
+    // scratch: adjoints of q_d and g_d per axis, the pressure side's gradient term
+    const size_t n_scratch = 2 * (size_t)m->ndim + 1;
+    Buf scratch(n_scratch * vol * sizeof(R)), gacc(2 * vol * sizeof(double)),
         uacc(2 * n_user * sizeof(double));
     const size_t nG = (size_t)m->n_rcv * m->n_rec;
     Buf dG(nG * sizeof(R)), dA0(alpha0 ? n_user * (as_f64 ? 8 : 4) : 0);
     Buf dlut((size_t)m->n_classes * kDStride * sizeof(R)), zero(256);   // zero: step counter of the image steps
-    if (!lam.p || (one_kernel && !lam2.p) || !ck.p || !seg0.p || (n_ck > 1 && !seg1.p) || !fin.p || (!one_kernel && !scratch.p) || !gacc.p ||
-        !uacc.p || (nG && !dG.p) || (alpha0 && !dA0.p) || !dlut.p || !zero.p)
+    if (!lam.p || !ck.p || !seg0.p || (n_ck > 1 && !seg1.p) || !fin.p || !scratch.p || !gacc.p || !uacc.p || (nG && !dG.p) || (alpha0 && !dA0.p) || !dlut.p || !zero.p)
         return FW_ERR_NOMEM;
     ADJ_CK(cudaMemsetAsync(zero.p, 0, 256, s));
     ADJ_CK(cudaMemsetAsync(lam.p, 0, SB, s));
-    if (one_kernel) ADJ_CK(cudaMemsetAsync(lam2.p, 0, SB, s));
-    else ADJ_CK(cudaMemsetAsync(scratch.p, 0, 6 * vol * sizeof(R), s));
+    ADJ_CK(cudaMemsetAsync(scratch.p, 0, n_scratch * vol * sizeof(R), s));
     ADJ_CK(cudaMemsetAsync(gacc.p, 0, 2 * vol * sizeof(double), s));
     ADJ_CK(cudaMemsetAsync(uacc.p, 0, 2 * n_user * sizeof(double), s));
     // receiver weights in the field type
@@ -929,9 +570,8 @@ int gradient_impl(fw_medium *m, int n_steps, int K, const void *G, const void *a
 
     // ---- kernel arguments (pointers into images are set per step) ----
     AdjArgs<R> A{};
-    A.nx = m->NX; A.ny = m->NY; A.nz = m->NZ; A.px = m->px; A.nmech = m->nmech;
+    A.nx = m->NX; A.ny = m->NY; A.nz = m->NZ; A.px = m->px;
     A.plane = (long long)m->plane;
-    A.vol = (long long)vol;
     const double cm[4] = {1225.0 / 1024.0, -245.0 / 3072.0, 49.0 / 5120.0, -5.0 / 7168.0};
     A.c1 = R(cm[0] / m->dx); A.c2 = R(cm[1] / m->dx); A.c3 = R(cm[2] / m->dx); A.c4 = R(cm[3] / m->dx);
     A.dt = R(m->dt);
@@ -952,18 +592,20 @@ int gradient_impl(fw_medium *m, int n_steps, int K, const void *G, const void *a
         for (int k = 0; k < m->nmech; ++k) S.lpsi2[k] = reinterpret_cast<R *>(L + off(m->psi2[k]));
         return S;
     };
-    A.in = state_in(lam.p);
-    A.out = one_kernel ? state_in(lam2.p) : A.in;
+    A.L = state_in(lam.p);
+    R *next = static_cast<R *>(scratch.p);
     for (int ax = 0; ax < 3; ++ax) {
-        A.ax_on[ax] = m->v[ax] != nullptr;
         const bool layer = m->psi1p[ax] != nullptr;
         A.pdh[ax] = layer ? static_cast<const R *>(m->prof[ax][0]) : nullptr;
         A.pah[ax] = layer ? static_cast<const R *>(m->prof[ax][1]) : nullptr;
         A.pdi[ax] = layer ? static_cast<const R *>(m->prof[ax][2]) : nullptr;
         A.pai[ax] = layer ? static_cast<const R *>(m->prof[ax][3]) : nullptr;
-        A.Q[ax] = one_kernel ? nullptr : static_cast<R *>(scratch.p) + ax * vol;
-        A.Gd[ax] = one_kernel ? nullptr : static_cast<R *>(scratch.p) + (3 + ax) * vol;
+        if (!m->v[ax]) continue;
+        A.Q[ax] = next;
+        A.Gd[ax] = next + vol;
+        next += 2 * vol;
     }
+    A.gsp = next;
     A.kdt = static_cast<const R *>(m->kdt);
     A.rho = static_cast<const R *>(m->rho);
     A.cls = m->cls;
@@ -971,9 +613,21 @@ int gradient_impl(fw_medium *m, int n_steps, int K, const void *G, const void *a
     A.dlut = static_cast<const R *>(dlut.p);
     A.gk = static_cast<double *>(gacc.p);
     A.gs = static_cast<double *>(gacc.p) + vol;
-    const dim3 pgrid((unsigned)((m->NX + 255) / 256), (unsigned)m->NY, (unsigned)m->NZ);   // one thread per point
     const double inv_dxd = 1.0 / std::pow(m->dx, m->ndim);
-    ADJ_CK(launch_reverse<R>(A, m->ndim, m->nmech, pgrid, s, true));
+    // trace column of time step it, -1 where it is not recorded
+    auto column = [m](long long it) {
+        return m->n_rcv > 0 && it % m->decim == 0 && it / m->decim < m->n_rec ? (int)(it / m->decim) : -1;
+    };
+    // source gradient of step it (-1: none) and receivers' adjoints of trace column col
+    auto adjoint_io = [&](long long it, int col) {
+        const int n_io = m->n_src + (col >= 0 ? m->n_rcv : 0);
+        if (n_io <= 0 || (col < 0 && (it < 0 || it >= m->wave_len))) return;
+        k_adj_io<R><<<(n_io + 255) / 256, 256, 0, s>>>(A.L.lp, m->src_idx, static_cast<const R *>(m->waves), m->wave_of,
+                                                       m->wave_len, (int)it, m->n_src, m->src_rcv, m->rcv_idx,
+                                                       m->rcv_src, static_cast<const R *>(dG.p), m->n_rcv, m->n_rec,
+                                                       col, inv_dxd, A.gk);
+    };
+    adjoint_io(-1, column(it0 + n_steps - 1));   // the last step's receivers
 
     // ---- reverse sweep, one checkpoint segment at a time ----
     // The recomputation of segment si - 1 (a side stream, into the other of two
@@ -1033,14 +687,6 @@ int gradient_impl(fw_medium *m, int n_steps, int K, const void *G, const void *a
         };
         for (int k = k1 - 1; k >= k0; --k) {
             const long long it = it0 + k;
-            const int col = (m->n_rcv > 0 && it % m->decim == 0 && it / m->decim < m->n_rec) ? (int)(it / m->decim) : -1;
-            if (col >= 0 || (m->n_src > 0 && it < m->wave_len)) {
-                const int n_io = m->n_src + (col >= 0 ? m->n_rcv : 0);
-                k_adj_io<R><<<(n_io + 255) / 256, 256, 0, s>>>(A.in.lp, m->src_idx, static_cast<const R *>(m->waves),
-                                                               m->wave_of, m->wave_len, (int)it, m->n_src, m->src_rcv,
-                                                               m->rcv_idx, m->rcv_src, static_cast<const R *>(dG.p),
-                                                               m->n_rcv, m->n_rec, col, inv_dxd, A.gk);
-            }
             const char *F = image(k - k0), *F1 = image(k - k0 + 1);
             A.fp = reinterpret_cast<const R *>(F + off(m->p));
             for (int ax = 0; ax < 3; ++ax) {
@@ -1050,8 +696,9 @@ int gradient_impl(fw_medium *m, int n_steps, int K, const void *G, const void *a
                     A.fpsi1[q][ax] = m->psi1[q][ax] ? reinterpret_cast<const R *>(F + off(m->psi1[q][ax])) : nullptr;
             }
             for (int q = 0; q < m->nmech; ++q) A.fpsi2[q] = reinterpret_cast<const R *>(F + off(m->psi2[q]));
-            ADJ_CK(launch_reverse<R>(A, m->ndim, m->nmech, pgrid, s));
-            if (one_kernel) std::swap(A.in, A.out);
+            ADJ_CK(launch_reverse<R>(A, m->ndim, m->nmech, 2, s));
+            adjoint_io(it, k > 0 ? column(it - 1) : -1);
+            ADJ_CK(launch_reverse<R>(A, m->ndim, m->nmech, 1, s));
         }
         ADJ_CK(cudaEventRecord(rev_done[si & 1], s));
         rev_recorded[si & 1] = true;

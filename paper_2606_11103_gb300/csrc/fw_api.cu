@@ -438,10 +438,9 @@ double psi_scale_of(const fw_medium *m, int side)
 }  // namespace fwgb
 namespace {
 
-// per-class coefficient table for the run's dt (Eqs. relaxation_a/b), with
-// the midpoint memory-variable update folded in (ceff, hb); the stored memory
-// variables of the gradient and divergence sides may be scaled (binary16
-// storage, psi_scale_of).
+// per-class coefficient table for the run's dt (Eqs. relaxation_a/b); the
+// stored memory variables of the gradient and divergence sides may be scaled
+// (binary16 storage, psi_scale_of).
 // FP32 media: the sweeps take 1/kappa as a pair of FP32 values, and the pair
 // carries the correction for the FP32 rounding of dt (velocity side) and of the
 // stencil weights (their gain on long waves, both sides).  In a homogeneous
@@ -468,29 +467,20 @@ std::vector<double> build_lut(const fw_medium *m)
         double *e = &t[c * kLutStride];
         e[0] = p.kappa1;
         e[1] = p.kappa2;
-        double sa1 = 0.0, sa2 = 0.0;   // sum a/2 per stretch
         for (int m = 0; m < p.n_mech; ++m) {
             double b1 = std::exp(-(p.d1[m] / p.kappa1 + p.alpha1[m]) * dt);
             double a1 = p.d1[m] / (p.kappa1 * (p.d1[m] + p.kappa1 * p.alpha1[m])) * (b1 - 1.0);
             double b2 = std::exp(-(p.d2[m] / p.kappa2 + p.alpha2[m]) * dt);
             double a2 = p.d2[m] / (p.kappa2 * (p.d2[m] + p.kappa2 * p.alpha2[m])) * (b2 - 1.0);
-            sa1 += 0.5 * a1;
-            sa2 += 0.5 * a2;
             e[kLutA1 + m] = a1 * sc1;
             e[kLutB1 + m] = b1;
-            e[kLutH1 + m] = 0.5 * (1.0 + b1) / sc1;
             e[kLutA2 + m] = a2 * sc2;
             e[kLutB2 + m] = b2;
-            e[kLutH2 + m] = 0.5 * (1.0 + b2) / sc2;
         }
-        e[2] = 1.0 / p.kappa1 + sa1;
-        e[3] = 1.0 / p.kappa2 + sa2;
-        e[kLutDk] = sa1;
-        e[kLutDk + 1] = sa2;
         const double ik[2] = {comp1 / p.kappa1, comp2 / p.kappa2};
         for (int k = 0; k < 2; ++k) {
-            e[kLutIk + k] = f32 ? double(float(ik[k])) : ik[k];
-            e[kLutIk + 2 + k] = ik[k] - e[kLutIk + k];
+            e[kLutIk1 + 2 * k] = f32 ? double(float(ik[k])) : ik[k];
+            e[kLutIk1 + 2 * k + 1] = ik[k] - e[kLutIk1 + 2 * k];
         }
     }
     return t;

@@ -29,15 +29,12 @@ int nelder_mead(int n, double *x, const double *lo, const double *hi,
                 double xatol, double fatol, double *fmin, int *n_iter, int *n_eval);
 
 // ---- device layout ---------------------------------------------------------
-constexpr int kLutStride = 36;   // values per class in the coefficient table
-// table block offsets (in values): 0 kappa1, 1 kappa2, 2 ceff1, 3 ceff2,
-// 4.. a1[4], 8.. b1[4], 12.. hb1[4], 16.. a2[4], 20.. b2[4], 24.. hb2[4],
-// 28 sum a1/2, 29 sum a2/2 (= ceff - 1/kappa, the part the layer ramp scales),
-// 30 1/kappa1, 31 1/kappa2, 32, 33 what the rounding of 30, 31 left off (FP32
-// media; both with the known rounding of the global factors taken back, see
-// build_lut).  The sweeps use a, b and 30..33, the adjoint the others.
-constexpr int kLutA1 = 4, kLutB1 = 8, kLutH1 = 12, kLutA2 = 16, kLutB2 = 20, kLutH2 = 24, kLutDk = 28,
-              kLutIk = 30;
+constexpr int kLutStride = 24;   // values per class in the coefficient table
+// table block offsets (in values): 0 kappa1, 1 kappa2, 4.. a1[4], 8.. b1[4],
+// 12.. a2[4], 16.. b2[4], 20 1/kappa1, 21 what its rounding left off, 22, 23
+// the same of kappa2 (the remainders: FP32 media; both with the known rounding
+// of the global factors taken back, see build_lut)
+constexpr int kLutA1 = 4, kLutB1 = 8, kLutA2 = 12, kLutB2 = 16, kLutIk1 = 20, kLutIk2 = 22;
 
 struct Monitor {
     unsigned int max_bits;   // bits of max |p| (non-negative float)

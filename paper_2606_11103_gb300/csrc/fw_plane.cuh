@@ -184,7 +184,7 @@ k_velocity_plane(const __grid_constant__ VelArgs<R, SS, SP> A, int gx)
     uint16_t cls4[4];
     quad_classes(cl, cls4);
     QuadCoef<R, NM> C;
-    C.load(A.lut, cls4, kLutA1, kLutB1, kLutIk);
+    C.load(A.lut, cls4, kLutA1, kLutB1, kLutIk1);
 
     R g[3][4], dtr[3][4];
     if (TS) {   // the time-space stencil (see vel_gradient_ts)
@@ -249,7 +249,7 @@ k_pressure_plane(const __grid_constant__ PresArgs<R, SS, SP> A, int gx)
         uint16_t cls4[4];
         quad_classes(cl, cls4);
         QuadCoef<R, NM> C;
-        C.load(A.lut, cls4, kLutA2, kLutB2, kLutIk + 1);
+        C.load(A.lut, cls4, kLutA2, kLutB2, kLutIk2);
         R qd[3][4];
         if (TS) {   // the time-space stencil (see pres_divergence_ts)
             R rh[4], up[4], dn[4];
@@ -417,7 +417,7 @@ k_velocity_tiles(const __grid_constant__ VelArgs<float, float, SP> A, const __gr
         uint16_t cls4[4];
         quad_classes(cl, cls4);
         if (cl.x != key.x || cl.y != key.y) {
-            C.load(A.lut, cls4, kLutA1, kLutB1, kLutIk);
+            C.load(A.lut, cls4, kLutA1, kLutB1, kLutIk1);
             key = cl;
         }
         float q[8][4], w[12], own[4], nx1[4], nz1[4], g[3][4], dtr[3][4];
@@ -507,7 +507,7 @@ k_pressure_tiles(const __grid_constant__ PresArgs<float, float, SP> A, const __g
         uint16_t cls4[4];
         quad_classes(cl, cls4);
         if (cl.x != key.x || cl.y != key.y) {
-            C.load(A.lut, cls4, kLutA2, kLutB2, kLutIk + 1);
+            C.load(A.lut, cls4, kLutA2, kLutB2, kLutIk2);
             key = cl;
         }
         float qz[8][4], w[12], kd[4], bd[4], pv[4], ps[NM][4], qd[3][4];
