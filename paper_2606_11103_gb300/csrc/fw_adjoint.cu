@@ -31,7 +31,7 @@
 // Gradients accumulate in FP64.
 // The linear system only (no nonlinear factor); FP32 and FP64 media.
 #include "fw_internal.h"
-#include "fw_kernels.cuh"
+#include "fw_launch.cuh"
 
 #include <algorithm>
 #include <cmath>
@@ -41,8 +41,8 @@ namespace fwgb {
 void *device_alloc(size_t bytes);
 void device_free(void *p);
 size_t state_image_bytes(const fw_medium *m);
-cudaError_t image_step_f32(const fw_medium *m, const StepImages &im, const int *zero, int it, cudaStream_t s);
-cudaError_t image_step_f64(const fw_medium *m, const StepImages &im, const int *zero, int it, cudaStream_t s);
+cudaError_t image_step_f32(const fw_medium *m, const StepImages &im, const int *zero, int it, bool pdl, cudaStream_t s);
+cudaError_t image_step_f64(const fw_medium *m, const StepImages &im, const int *zero, int it, bool pdl, cudaStream_t s);
 }  // namespace fwgb
 
 using namespace fwgb;
@@ -181,8 +181,14 @@ template <typename R, int DIM, int NM>
 __global__ void __launch_bounds__(32 * kAdjRows, sizeof(R) == 4 ? 4 : 1) k_adj_pressure(const __grid_constant__ AdjArgs<R> A)
 {
     const AdjPos P = adj_pos<R, DIM>(A);
-    if (!P.on) return;
+    uint16_t cls[4];
     R lp[4], kd[4], q[3][4], div[4], d[4];
+    if (P.on) {
+        quad_classes(__ldg(reinterpret_cast<const uint2 *>(A.cls + P.i)), cls);
+        Io<R>::ldg(A.kdt + P.i, kd);
+    }
+    pdl_wait();
+    if (!P.on) return;
     Io<R>::ld(A.L.lp + P.i, lp);
     adj_diff<R, 0, false>(A, P, A.Gd[0], d);
 #pragma unroll
@@ -195,15 +201,11 @@ __global__ void __launch_bounds__(32 * kAdjRows, sizeof(R) == 4 ? 4 : 1) k_adj_p
     adj_diff<R, 2, false>(A, P, A.Gd[2], d);
 #pragma unroll
     for (int e = 0; e < 4; ++e) lp[e] = P.c[0] + e < A.nx ? lp[e] - (div[e] + d[e]) : R(0);
-    Io<R>::st(A.L.lp + P.i, lp);
     adj_diff<R, 0, false>(A, P, A.fv1[0], q[0]);
     adj_diff<R, 2, false>(A, P, A.fv1[2], q[2]);
     if (DIM == 3) adj_diff<R, 1, false>(A, P, A.fv1[1], q[1]);
 #pragma unroll
     for (int e = 0; e < 4; ++e) div[e] = DIM == 3 ? q[0][e] + q[2][e] + q[1][e] : q[0][e] + q[2][e];
-    Io<R>::ldg(A.kdt + P.i, kd);
-    uint16_t cls[4];
-    quad_classes(__ldg(reinterpret_cast<const uint2 *>(A.cls + P.i)), cls);
     R ln[NM][4], old[NM][4];
 #pragma unroll
     for (int m = 0; m < NM; ++m) {
@@ -232,6 +234,8 @@ __global__ void __launch_bounds__(32 * kAdjRows, sizeof(R) == 4 ? 4 : 1) k_adj_p
         stp[e] = fma(C.ik, div[e], fma(C.il, div[e], R(0.5) * mem));
         gsp[e] = gs;
     }
+    pdl_launch();
+    Io<R>::st(A.L.lp + P.i, lp);
 #pragma unroll
     for (int m = 0; m < NM; ++m) Io<R>::st(A.L.lpsi2[m] + P.i, ln[m]);
     Io<R>::st(A.gsp + P.i, gsp);
@@ -334,11 +338,14 @@ template <typename R, int DIM, int NM>
 __global__ void __launch_bounds__(32 * kAdjRows, sizeof(R) == 4 ? 4 : 1) k_adj_velocity(const __grid_constant__ AdjArgs<R> A)
 {
     const AdjPos P = adj_pos<R, DIM>(A);
-    if (!P.on) return;
     uint16_t cls[4];
-    quad_classes(__ldg(reinterpret_cast<const uint2 *>(A.cls + P.i)), cls);
     R own[4], gs[4], rr[4] = {R(1), R(1), R(1), R(1)};
-    Io<R>::ldg(A.rho + P.i, own);
+    if (P.on) {
+        quad_classes(__ldg(reinterpret_cast<const uint2 *>(A.cls + P.i)), cls);
+        Io<R>::ldg(A.rho + P.i, own);
+    }
+    pdl_wait();
+    if (!P.on) return;
     Io<R>::ld(A.gsp + P.i, gs);
     if (adj_in_layer<R, DIM>(A, P, 0) || adj_in_layer<R, DIM>(A, P, 1) || adj_in_layer<R, DIM>(A, P, 2))
 #pragma unroll
@@ -346,6 +353,7 @@ __global__ void __launch_bounds__(32 * kAdjRows, sizeof(R) == 4 ? 4 : 1) k_adj_v
     adj_velocity_axis<R, DIM, NM, 0>(A, P, cls, own, rr, gs);
     if (DIM == 3) adj_velocity_axis<R, DIM, NM, 1>(A, P, cls, own, rr, gs);
     adj_velocity_axis<R, DIM, NM, 2>(A, P, cls, own, rr, gs);
+    pdl_launch();
     const double g[4] = {double(gs[0]), double(gs[1]), double(gs[2]), double(gs[3])};
     add4(A.gs + P.i, g);
 }
@@ -361,6 +369,8 @@ __global__ void k_adj_io(R *lp, const long long *src_idx, const R *waves, const 
                          int n_src, const int *src_rcv, const long long *rcv_idx, const int *rcv_src, const R *G,
                          int n_rcv, int n_col, int col, double inv_dxd, double *gk)
 {
+    pdl_launch();
+    pdl_wait();
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t < n_src) {
         const long long k = src_idx[t];
@@ -420,27 +430,26 @@ __global__ void k_grad_out(const double *uc, const double *us, const float *a0f,
 }
 
 template <typename R, int DIM, int NM>
-cudaError_t launch_reverse_n(const AdjArgs<R> &A, int side, cudaStream_t s)
+cudaError_t launch_reverse_n(const AdjArgs<R> &A, int side, bool pdl, cudaStream_t s)
 {
     const unsigned gx = (unsigned)(A.nx + 127) / 128;
     const unsigned rows = DIM == 3 ? (unsigned)(A.ny + kAdjRows - 1) / kAdjRows * (unsigned)A.nz
                                    : (unsigned)(A.nz + kAdjRows - 1) / kAdjRows;
-    if (side == 2) k_adj_pressure<R, DIM, NM><<<gx * rows, dim3(32, kAdjRows), 0, s>>>(A);
-    else k_adj_velocity<R, DIM, NM><<<gx * rows, dim3(32, kAdjRows), 0, s>>>(A);
-    return cudaGetLastError();
+    return launch_kernel(side == 2 ? k_adj_pressure<R, DIM, NM> : k_adj_velocity<R, DIM, NM>, dim3(gx * rows),
+                         dim3(32, kAdjRows), 0, s, pdl, A);
 }
 
 // one half of a reverse step (side 2: pressure, 1: velocity); instances per
 // dimension and number of mechanisms (their loops unroll)
 template <typename R>
-cudaError_t launch_reverse(const AdjArgs<R> &A, int ndim, int nmech, int side, cudaStream_t s)
+cudaError_t launch_reverse(const AdjArgs<R> &A, int ndim, int nmech, int side, bool pdl, cudaStream_t s)
 {
     const bool d3 = ndim == 3;
     switch (nmech) {
-    case 1: return d3 ? launch_reverse_n<R, 3, 1>(A, side, s) : launch_reverse_n<R, 2, 1>(A, side, s);
-    case 2: return d3 ? launch_reverse_n<R, 3, 2>(A, side, s) : launch_reverse_n<R, 2, 2>(A, side, s);
-    case 3: return d3 ? launch_reverse_n<R, 3, 3>(A, side, s) : launch_reverse_n<R, 2, 3>(A, side, s);
-    default: return d3 ? launch_reverse_n<R, 3, 4>(A, side, s) : launch_reverse_n<R, 2, 4>(A, side, s);
+    case 1: return d3 ? launch_reverse_n<R, 3, 1>(A, side, pdl, s) : launch_reverse_n<R, 2, 1>(A, side, pdl, s);
+    case 2: return d3 ? launch_reverse_n<R, 3, 2>(A, side, pdl, s) : launch_reverse_n<R, 2, 2>(A, side, pdl, s);
+    case 3: return d3 ? launch_reverse_n<R, 3, 3>(A, side, pdl, s) : launch_reverse_n<R, 2, 3>(A, side, pdl, s);
+    default: return d3 ? launch_reverse_n<R, 3, 4>(A, side, pdl, s) : launch_reverse_n<R, 2, 4>(A, side, pdl, s);
     }
 }
 
@@ -619,15 +628,17 @@ int gradient_impl(fw_medium *m, int n_steps, int K, const void *G, const void *a
         return m->n_rcv > 0 && it % m->decim == 0 && it / m->decim < m->n_rec ? (int)(it / m->decim) : -1;
     };
     // source gradient of step it (-1: none) and receivers' adjoints of trace column col
+    cudaError_t e_io = cudaSuccess;
     auto adjoint_io = [&](long long it, int col) {
         const int n_io = m->n_src + (col >= 0 ? m->n_rcv : 0);
         if (n_io <= 0 || (col < 0 && (it < 0 || it >= m->wave_len))) return;
-        k_adj_io<R><<<(n_io + 255) / 256, 256, 0, s>>>(A.L.lp, m->src_idx, static_cast<const R *>(m->waves), m->wave_of,
-                                                       m->wave_len, (int)it, m->n_src, m->src_rcv, m->rcv_idx,
-                                                       m->rcv_src, static_cast<const R *>(dG.p), m->n_rcv, m->n_rec,
-                                                       col, inv_dxd, A.gk);
+        e_io = launch_kernel(k_adj_io<R>, dim3((n_io + 255) / 256), dim3(256), 0, s, true, A.L.lp, m->src_idx,
+                             static_cast<const R *>(m->waves), m->wave_of, m->wave_len, (int)it, m->n_src, m->src_rcv,
+                             m->rcv_idx, m->rcv_src, static_cast<const R *>(dG.p), m->n_rcv, m->n_rec, col, inv_dxd,
+                             A.gk);
     };
     adjoint_io(-1, column(it0 + n_steps - 1));   // the last step's receivers
+    ADJ_CK(e_io);
 
     // ---- reverse sweep, one checkpoint segment at a time ----
     // The recomputation of segment si - 1 (a side stream, into the other of two
@@ -654,8 +665,8 @@ int gradient_impl(fw_medium *m, int n_steps, int K, const void *G, const void *a
             char *wr = segs[si & 1] + (size_t)(k - k0) * SB;
             const StepImages im{rd, (long long)(wr - rd)};
             const int itk = (int)(it0 + k);
-            if ((sizeof(R) == 8 ? image_step_f64(m, im, static_cast<const int *>(zero.p), itk, ss.side)
-                                : image_step_f32(m, im, static_cast<const int *>(zero.p), itk, ss.side)) != cudaSuccess)
+            if ((sizeof(R) == 8 ? image_step_f64(m, im, static_cast<const int *>(zero.p), itk, k > k0, ss.side)
+                                : image_step_f32(m, im, static_cast<const int *>(zero.p), itk, k > k0, ss.side)) != cudaSuccess)
                 return FW_ERR_CUDA;
             rd = wr;
         }
@@ -696,9 +707,11 @@ int gradient_impl(fw_medium *m, int n_steps, int K, const void *G, const void *a
                     A.fpsi1[q][ax] = m->psi1[q][ax] ? reinterpret_cast<const R *>(F + off(m->psi1[q][ax])) : nullptr;
             }
             for (int q = 0; q < m->nmech; ++q) A.fpsi2[q] = reinterpret_cast<const R *>(F + off(m->psi2[q]));
-            ADJ_CK(launch_reverse<R>(A, m->ndim, m->nmech, 2, s));
+            // a segment's first kernel follows an event of the side stream: no early start
+            ADJ_CK(launch_reverse<R>(A, m->ndim, m->nmech, 2, k < k1 - 1, s));
             adjoint_io(it, k > 0 ? column(it - 1) : -1);
-            ADJ_CK(launch_reverse<R>(A, m->ndim, m->nmech, 1, s));
+            ADJ_CK(e_io);
+            ADJ_CK(launch_reverse<R>(A, m->ndim, m->nmech, 1, true, s));
         }
         ADJ_CK(cudaEventRecord(rev_done[si & 1], s));
         rev_recorded[si & 1] = true;

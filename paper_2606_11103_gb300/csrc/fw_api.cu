@@ -19,8 +19,9 @@ cudaError_t sweeps_f32(const fw_medium *m, cudaStream_t s, int which);
 cudaError_t sweeps_bf16(const fw_medium *m, cudaStream_t s, int which);
 cudaError_t sweeps_f16(const fw_medium *m, cudaStream_t s, int which);
 cudaError_t sweeps_f64(const fw_medium *m, cudaStream_t s, int which);
-cudaError_t io_f32(const fw_medium *m, int j, cudaStream_t s);
-cudaError_t io_f64(const fw_medium *m, int j, cudaStream_t s);
+cudaError_t io_f32(const fw_medium *m, int j, bool pdl, cudaStream_t s);
+cudaError_t io_f64(const fw_medium *m, int j, bool pdl, cudaStream_t s);
+cudaError_t launch_advance(int *d_it, int n, bool pdl, cudaStream_t s);
 void noalloc_prepare();
 using EncodeTiledFn = CUresult (*)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
                                    const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
@@ -571,23 +572,22 @@ cudaError_t launch_sweep(const fw_medium *m, cudaStream_t s, int which)
     }
 }
 
-cudaError_t launch_io_any(const fw_medium *m, int j, cudaStream_t s)
+cudaError_t launch_io_any(const fw_medium *m, int j, bool pdl, cudaStream_t s)
 {
-    return m->storage == FW_STORE_F64 ? io_f64(m, j, s) : io_f32(m, j, s);
+    return m->storage == FW_STORE_F64 ? io_f64(m, j, pdl, s) : io_f32(m, j, pdl, s);
 }
 
 cudaError_t launch_step(const fw_medium *m, int j, cudaStream_t s)
 {
     cudaError_t e = launch_sweep(m, s, 3);
     if (e != cudaSuccess) return e;
-    return launch_io_any(m, j, s);
+    return launch_io_any(m, j, true, s);
 }
 
 int enqueue_steps(fw_medium *m, int n, cudaStream_t s)
 {
     for (int j = 0; j < n; ++j) FW_CK(launch_step(m, j, s));
-    k_advance<<<1, 1, 0, s>>>(m->d_it, n);
-    FW_CK(cudaGetLastError());
+    FW_CK(launch_advance(m->d_it, n, true, s));
     return FW_OK;
 }
 
@@ -1213,16 +1213,15 @@ int fw_step_timed(fw_medium *m, int n_steps, void *stream, double *ms_velocity, 
     int rc = FW_OK;
     int launches = 0;
     for (int j = 0; j < n_steps && rc == FW_OK; ++j) {
-        if (cudaEventRecord(ev[3 * j], s) != cudaSuccess || launch_sweep(m, s, 1) != cudaSuccess ||
-            cudaEventRecord(ev[3 * j + 1], s) != cudaSuccess || launch_sweep(m, s, 2) != cudaSuccess ||
-            cudaEventRecord(ev[3 * j + 2], s) != cudaSuccess || launch_io_any(m, j, s) != cudaSuccess)
+        if (cudaEventRecord(ev[3 * j], s) != cudaSuccess || launch_sweep(m, s, 1 | 8) != cudaSuccess ||
+            cudaEventRecord(ev[3 * j + 1], s) != cudaSuccess || launch_sweep(m, s, 2 | 8) != cudaSuccess ||
+            cudaEventRecord(ev[3 * j + 2], s) != cudaSuccess || launch_io_any(m, j, false, s) != cudaSuccess)
             rc = FW_ERR_CUDA;
         launches += 2 + (m->n_src + m->n_rcv > 0);
     }
     if (rc == FW_OK) {
-        k_advance<<<1, 1, 0, s>>>(m->d_it, n_steps);
         launches += 1;
-        if (cudaGetLastError() != cudaSuccess || cudaEventRecord(ev[3 * (size_t)n_steps], s) != cudaSuccess ||
+        if (launch_advance(m->d_it, n_steps, false, s) != cudaSuccess || cudaEventRecord(ev[3 * (size_t)n_steps], s) != cudaSuccess ||
             cudaEventSynchronize(ev[3 * (size_t)n_steps]) != cudaSuccess)
             rc = FW_ERR_CUDA;
     }

@@ -11,6 +11,24 @@
 
 namespace fwgb {
 
+// Launch with or without the programmatic attribute (pdl_wait in the kernels).
+// Left out after an event of another stream and where events time each kernel.
+template <typename... P, typename... A>
+cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, bool pdl, A &&...args)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = pdl ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // rows of the 3D CTA tiles (tuning knobs, measured best): the velocity sweep
 // runs two 128x4 CTAs per SM, the pressure sweep three 128x4 CTAs per SM
 #ifndef FWGB_VEL3_BY
@@ -208,7 +226,7 @@ PresArgs<R, SS, SP> pres_args(const fw_medium *m, const StepImages *im)
 // Sweeps of one dimension, mechanism count and time scheme.  which: bit 0 =
 // velocity sweep, bit 1 = pressure sweep, bit 2 = only opt the instances into
 // their dynamic shared memory (done once at medium creation, outside any
-// stream capture).  im (may be null): a step from one state image into another
+// stream capture), bit 3 = launches without the programmatic attribute.  im (may be null): a step from one state image into another
 // (StepImages) instead of the in-place step of the medium's own state.
 // 2D FP32-state grids from kTileMin tiles on take the staged sweeps, in runs of
 // two tiles per CTA, of four from kTileLong tiles on; smaller grids, FP64 media
@@ -238,9 +256,13 @@ cudaError_t launch_tiles(const fw_medium *m, cudaStream_t s, int which, int gx, 
     const dim3 block(32, kTileH);
     const int run = n_tiles >= kTileLong ? 4 : 2;
     const int rows = n_tiles / gx, ctas = gx * ((rows + run - 1) / run);
-    if (which & 1) kv<<<ctas, block, bv, s>>>(vel_args<float, float, SP, NM>(m, nullptr), m->vel_maps, gx, run, rows);
-    if (which & 2) kp<<<ctas, block, bp, s>>>(pres_args<float, float, SP, NM>(m, nullptr), m->pres_maps, gx, run, rows);
-    return cudaGetLastError();
+    const bool pdl = !(which & 8);
+    cudaError_t e = cudaSuccess;
+    if (which & 1)
+        e = launch_kernel(kv, dim3(ctas), block, bv, s, pdl, vel_args<float, float, SP, NM>(m, nullptr), m->vel_maps, gx, run, rows);
+    if (e == cudaSuccess && (which & 2))
+        e = launch_kernel(kp, dim3(ctas), block, bp, s, pdl, pres_args<float, float, SP, NM>(m, nullptr), m->pres_maps, gx, run, rows);
+    return e;
 }
 
 template <typename R, typename SS, typename SP, int NM, bool TS>
@@ -254,13 +276,16 @@ cudaError_t launch_2d(const fw_medium *m, cudaStream_t s, int which, const StepI
     }
     if (which & 4) return cudaSuccess;
     const dim3 grid((unsigned)gx * (unsigned)((m->NZ + kPlaneBY - 1) / kPlaneBY)), block(32, kPlaneBY);
-    if (which & 1) k_velocity_plane<R, SS, SP, NM, kPlaneBY, TS><<<grid, block, 0, s>>>(vel_args<R, SS, SP, NM>(m, im), gx);
-    if (which & 2) {
-        const auto pa = pres_args<R, SS, SP, NM>(m, im);
-        if (m->nonlinear) k_pressure_plane<R, SS, SP, NM, kPlaneBY, true, TS><<<grid, block, 0, s>>>(pa, gx);
-        else k_pressure_plane<R, SS, SP, NM, kPlaneBY, false, TS><<<grid, block, 0, s>>>(pa, gx);
-    }
-    return cudaGetLastError();
+    const bool pdl = !(which & 8);
+    cudaError_t e = cudaSuccess;
+    if (which & 1)
+        e = launch_kernel(k_velocity_plane<R, SS, SP, NM, kPlaneBY, TS>, grid, block, 0, s, pdl,
+                          vel_args<R, SS, SP, NM>(m, im), gx);
+    if (e == cudaSuccess && (which & 2))
+        e = launch_kernel(m->nonlinear ? k_pressure_plane<R, SS, SP, NM, kPlaneBY, true, TS>
+                                       : k_pressure_plane<R, SS, SP, NM, kPlaneBY, false, TS>,
+                          grid, block, 0, s, pdl, pres_args<R, SS, SP, NM>(m, im), gx);
+    return e;
 }
 
 template <typename R, typename SS, typename SP, int NM, bool TS, bool TMA>
@@ -285,12 +310,15 @@ cudaError_t launch_3d_as(const fw_medium *m, cudaStream_t s, int which, const St
         pm = m->pres_maps;
     }
     const int gx = (m->NX + 4 * BX - 1) / (4 * BX), gz = (m->NZ + m->zseg - 1) / m->zseg;
+    const bool pdl = !(which & 8);
+    cudaError_t e = cudaSuccess;
     if (which & 1)
-        kv<<<dim3(gx, (m->NY + BYV - 1) / BYV, gz), dim3(BX, BYV), LV::bytes, s>>>(vel_args<R, SS, SP, NM>(m, im), vm);
-    if (which & 2)
-        (m->nonlinear ? kpn : kp)<<<dim3(gx, (m->NY + BYP - 1) / BYP, gz), dim3(BX, BYP), LP::bytes, s>>>(
-            pres_args<R, SS, SP, NM>(m, im), pm);
-    return cudaGetLastError();
+        e = launch_kernel(kv, dim3(gx, (m->NY + BYV - 1) / BYV, gz), dim3(BX, BYV), LV::bytes, s, pdl,
+                          vel_args<R, SS, SP, NM>(m, im), vm);
+    if (e == cudaSuccess && (which & 2))
+        e = launch_kernel(m->nonlinear ? kpn : kp, dim3(gx, (m->NY + BYP - 1) / BYP, gz), dim3(BX, BYP), LP::bytes, s,
+                          pdl, pres_args<R, SS, SP, NM>(m, im), pm);
+    return e;
 }
 
 // The FP32-state sweeps stage their streams by TMA when the medium holds
@@ -337,30 +365,32 @@ cudaError_t launch_sweeps(const fw_medium *m, cudaStream_t s, int which, const S
 // counters are not used.  For the adjoint's recomputation: no copy of the
 // state per step, the medium's own state untouched.
 template <typename R, typename SS>
-cudaError_t launch_image_step(const fw_medium *m, const StepImages &im, const int *zero, int it, cudaStream_t s)
+cudaError_t launch_image_step(const fw_medium *m, const StepImages &im, const int *zero, int it, bool pdl, cudaStream_t s)
 {
-    cudaError_t e = launch_sweeps<R, SS, SS>(m, s, 3, &im);
+    cudaError_t e = cudaSuccess;
+    if (pdl) {
+        e = launch_sweeps<R, SS, SS>(m, s, 3, &im);
+    } else {                       // first kernel after an event of another stream
+        e = launch_sweeps<R, SS, SS>(m, s, 1 | 8, &im);
+        if (e == cudaSuccess) e = launch_sweeps<R, SS, SS>(m, s, 2, &im);
+    }
     if (e != cudaSuccess || m->n_src <= 0) return e;
     SS *p = reinterpret_cast<SS *>(const_cast<char *>(im.rd) + im.wofs +
                                    (static_cast<const char *>(m->p) - static_cast<const char *>(m->slab)));
-    k_sources<SS, R><<<(m->n_src + 255) / 256, 256, 0, s>>>(p, m->src_idx, static_cast<const R *>(m->src_gain),
-                                                           m->wave_of, static_cast<const R *>(m->waves),
-                                                           m->wave_len, m->n_src, zero, it, (long long)m->vol,
-                                                           m->mon);
-    return cudaGetLastError();
+    return launch_kernel(k_sources<SS, R>, dim3((m->n_src + 255) / 256), dim3(256), 0, s, true, p, m->src_idx,
+                         static_cast<const R *>(m->src_gain), m->wave_of, static_cast<const R *>(m->waves), m->wave_len,
+                         m->n_src, zero, it, (long long)m->vol, m->mon);
 }
 
 template <typename R, typename SS>
-cudaError_t launch_io(const fw_medium *m, int j, cudaStream_t s)
+cudaError_t launch_io(const fw_medium *m, int j, bool pdl, cudaStream_t s)
 {
     const int n = m->n_src + m->n_rcv;
     if (n <= 0) return cudaSuccess;
-    k_io<SS, R><<<(n + 255) / 256, 256, 0, s>>>(static_cast<SS *>(m->p), m->src_idx,
-                                                 static_cast<const R *>(m->src_gain), m->wave_of,
-                                                 static_cast<const R *>(m->waves), m->wave_len, m->n_src, m->src_rcv,
-                                                 m->rcv_idx, m->rcv_src, static_cast<SS *>(m->traces), m->n_rcv,
-                                                 m->n_rec, m->decim, m->d_it, j, (long long)m->vol, m->mon);
-    return cudaGetLastError();
+    return launch_kernel(k_io<SS, R>, dim3((n + 255) / 256), dim3(256), 0, s, pdl, static_cast<SS *>(m->p), m->src_idx,
+                         static_cast<const R *>(m->src_gain), m->wave_of, static_cast<const R *>(m->waves), m->wave_len,
+                         m->n_src, m->src_rcv, m->rcv_idx, m->rcv_src, static_cast<SS *>(m->traces), m->n_rcv, m->n_rec,
+                         m->decim, m->d_it, j, (long long)m->vol, m->mon);
 }
 
 }  // namespace fwgb

@@ -169,14 +169,16 @@ k_velocity_plane(const __grid_constant__ VelArgs<R, SS, SP> A, int gx)
 {
     const Geo<R> &G = A.g;
     const PlanePos P = plane_pos<BY>(G, gx);
-    if (!P.on) return;
+    if (!P.on) {
+        pdl_wait();
+        return;
+    }
     const long long row = P.row;
     const int x0 = P.x0, z = P.z;
 
-    R q[8][4], w[12], own[4], nx1[4], nz1[4];
+    // maps and tables first, then (after the wait) every stream of the quad
+    R q[8][4], w[12], own[4], nx1[4], nz1[4], vv[2][4], ps[2][NM][4];
     const uint2 cl = __ldg(reinterpret_cast<const uint2 *>(A.cls + row));
-    plane_rows(A.p, G, P, -3, q);
-    plane_row12(A.p, G, P, q[3], w);
     Io<SS>::ldg(A.rho + row, own);
     ld4_or_zero(A.rho + row + G.px, z + 1 < G.nz, nz1);
     nx1[0] = own[1]; nx1[1] = own[2]; nx1[2] = own[3];
@@ -185,6 +187,16 @@ k_velocity_plane(const __grid_constant__ VelArgs<R, SS, SP> A, int gx)
     quad_classes(cl, cls4);
     QuadCoef<R, NM> C;
     C.load(A.lut, cls4, kLutA1, kLutB1, kLutIk1);
+    pdl_wait();
+    pdl_launch();
+    plane_rows(A.p, G, P, -3, q);
+    plane_row12(A.p, G, P, q[3], w);
+#pragma unroll
+    for (int ax = 0; ax < 2; ++ax) {
+        Io<SS>::ld(A.v[2 * ax] + row, vv[ax]);
+#pragma unroll
+        for (int m = 0; m < NM; ++m) Io<SP>::ld(A.psi[m][2 * ax] + row, ps[ax][m]);
+    }
 
     R g[3][4], dtr[3][4];
     if (TS) {   // the time-space stencil (see vel_gradient_ts)
@@ -205,11 +217,8 @@ k_velocity_plane(const __grid_constant__ VelArgs<R, SS, SP> A, int gx)
     if (in[0] || in[2]) plane_ramp(G, P, rr);
 #pragma unroll
     for (int ax = 0; ax < 3; ax += 2) {
-        R vv[4], ps[NM][4], stv[4];
-        Io<SS>::ld(A.v[ax] + row, vv);
-#pragma unroll
-        for (int m = 0; m < NM; ++m) Io<SP>::ld(A.psi[m][ax] + row, ps[m]);
-        quad_stretch<R, NM>(C, g[ax], rr, G.hs1, ps, stv);
+        R(&v)[4] = vv[ax / 2], (&pa)[NM][4] = ps[ax / 2], stv[4];
+        quad_stretch<R, NM>(C, g[ax], rr, G.hs1, pa, stv);
         if (in[ax]) {
             R pp[4], a[4], b[4];
             Io<SS>::ld(A.psip[ax] + row, pp);
@@ -218,10 +227,10 @@ k_velocity_plane(const __grid_constant__ VelArgs<R, SS, SP> A, int gx)
             Io<SS>::st(wr_at(A.psip[ax] + row, A.wofs), pp);
         }
 #pragma unroll
-        for (int h = 0; h < 2; ++h) unpair(vv, h, p_fma(pair(dtr[ax], h), pair(stv, h), pair(vv, h)));
-        Io<SS>::st(wr_at(A.v[ax] + row, A.wofs), vv);
+        for (int h = 0; h < 2; ++h) unpair(v, h, p_fma(pair(dtr[ax], h), pair(stv, h), pair(v, h)));
+        Io<SS>::st(wr_at(A.v[ax] + row, A.wofs), v);
 #pragma unroll
-        for (int m = 0; m < NM; ++m) Io<SP>::st(wr_at(A.psi[m][ax] + row, A.wofs), ps[m]);
+        for (int m = 0; m < NM; ++m) Io<SP>::st(wr_at(A.psi[m][ax] + row, A.wofs), pa[m]);
     }
 }
 
@@ -233,23 +242,27 @@ k_pressure_plane(const __grid_constant__ PresArgs<R, SS, SP> A, int gx)
     const Geo<R> &G = A.g;
     const PlanePos P = plane_pos<BY>(G, gx);
     PMax<R> pmax;
-    if (P.on) {
+    if (!P.on) {
+        pdl_wait();
+    } else {
         const long long row = P.row;
         const int x0 = P.x0, z = P.z;
         R qz[8][4], w[12], own[4], kd[4], bd[4], pv[4], ps[NM][4];
         const uint2 cl = __ldg(reinterpret_cast<const uint2 *>(A.cls + row));
-        plane_rows(A.v[2], G, P, -4, qz);
-        Io<SS>::ldg(A.v[0] + row, own);
-        plane_row12(A.v[0], G, P, own, w);
         Io<SS>::ldg(A.kdt + row, kd);
         if (NL) Io<SS>::ldg(A.b2dt + row, bd);
-        Io<SS>::ld(A.p + row, pv);
-#pragma unroll
-        for (int m = 0; m < NM; ++m) Io<SP>::ld(A.psi[m] + row, ps[m]);
         uint16_t cls4[4];
         quad_classes(cl, cls4);
         QuadCoef<R, NM> C;
         C.load(A.lut, cls4, kLutA2, kLutB2, kLutIk2);
+        pdl_wait();
+        pdl_launch();
+        plane_rows(A.v[2], G, P, -4, qz);
+        Sm<SS>::ld(A.v[0] + row, own);
+        plane_row12(A.v[0], G, P, own, w);
+        Io<SS>::ld(A.p + row, pv);
+#pragma unroll
+        for (int m = 0; m < NM; ++m) Io<SP>::ld(A.psi[m] + row, ps[m]);
         R qd[3][4];
         if (TS) {   // the time-space stencil (see pres_divergence_ts)
             R rh[4], up[4], dn[4];
@@ -355,11 +368,13 @@ __device__ __forceinline__ void walk_tiles(unsigned char *smem, int gx, int run,
         mbar_expect_tx(bars + i % NS, TX);
         load(xb, (r0 + i) * kTileH, smem + (i % NS) * STAGE, bars + i % NS);
     };
+    pdl_wait();
     for (int i = 0; i < NS - 1; ++i) issue(i);
     bool timed_out = false;
     for (int i = 0; i < n; ++i) {
         if (i > 0) __syncthreads();        // tile i - 1 is done with the stage that tile i + NS - 1 takes
         issue(i + NS - 1);
+        if (i + 1 == n) pdl_launch();
         body(xb, (r0 + i) * kTileH, smem + (i % NS) * STAGE, [&] {
             if (!timed_out && !mbar_wait_bounded(bars + i % NS, (unsigned)(i / NS) & 1u)) timed_out = true;
         });
