@@ -29,16 +29,15 @@ cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, dim3 block, size_t sm
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
-// rows of the 3D CTA tiles (tuning knobs, measured best): the velocity sweep
-// runs two 128x4 CTAs per SM, the pressure sweep three 128x4 CTAs per SM
-#ifndef FWGB_VEL3_BY
-#define FWGB_VEL3_BY 4
-#endif
-#ifndef FWGB_PRES3_BY
-#define FWGB_PRES3_BY 4
-#endif
+// 3D CTA tiles: 64 x 8 points in FP32 (a quad per thread, 128 threads), two CTAs
+// of the velocity sweep and three of the pressure sweep per SM; 64 x 4 in FP64.
+// Against 128 x 4 the halo of p per plane is 15 x 72 instead of 11 x 136
+// points and a row's last tile holds at most 63 idle columns; us per step,
+// 128 x 4 / 64 x 8 / 32 x 16: 128^3 87.9 / 84.2 / 84.1, 231x187x301 383 / 354 /
+// 360, 256^3 508 / 504 / 514, 256^3 binary16 391 / 374, 256^3 time-space 647 /
+// 623, 512^3 3822 / 3826.
 template <typename R> struct Tile3 {
-    static constexpr int BX = sizeof(R) == 8 ? 16 : 32, BYV = FWGB_VEL3_BY, BYP = FWGB_PRES3_BY;
+    static constexpr int BX = 16, BYV = sizeof(R) == 8 ? 4 : 8, BYP = BYV;
 };
 constexpr int kPlaneBY = 4;   // rows per CTA of the unstaged 2D sweeps
 

@@ -328,7 +328,6 @@ template <typename SP, int NM, bool TS> struct VelTile {
     static constexpr size_t o_sp = o_kv + (TS ? kTileN * 4 : 0);
     static constexpr size_t o_sr = o_sp + pad128(SW * SH * 4);
     static constexpr size_t stage = o_sr + pad128(RW * (kTileH + 1) * 4);
-    static constexpr unsigned tx = (unsigned)(o_sp + (SW * SH + RW * (kTileH + 1)) * 4);   // bytes the copies deliver
 };
 
 template <typename SP, int NM, bool NL, bool TS> struct PresTile {
@@ -342,21 +341,20 @@ template <typename SP, int NM, bool NL, bool TS> struct PresTile {
     static constexpr size_t o_vx = o_cls + kTileN * 2;
     static constexpr size_t o_vz = o_vx + pad128(XW * XH * 4);
     static constexpr size_t stage = o_vz + pad128(ZW * ZH * 4);
-    static constexpr unsigned tx = (unsigned)(o_vx + (XW * XH + ZW * ZH) * 4);
 };
 
 // The walk of a CTA over its run of tiles (gx strips, n_rows tiles per strip):
-// load(position, stage, barrier) issues a tile's copies from one thread NS - 1
-// tiles ahead, body(position, stage, wait) computes it in all.  Waits are
+// load(warp, position, stage, barrier) arms the barrier with the bytes of the
+// warp's share of a tile's copies and issues them NS - 1 tiles ahead, body(position, stage, wait) computes it in all.  Waits are
 // bounded; after a timeout the sweep is flagged on the monitor.
-template <int NS, size_t STAGE, unsigned TX, typename Load, typename Body>
+template <int NS, size_t STAGE, typename Load, typename Body>
 __device__ __forceinline__ void walk_tiles(unsigned char *smem, int gx, int run, int n_rows, Monitor *mon, const Load &load,
                                            const Body &body)
 {
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + NS * STAGE);
-    const bool lead = threadIdx.x == 0 && threadIdx.y == 0;
-    if (lead) {
-        for (int b = 0; b < NS; ++b) mbar_init(bars + b, 1);
+    const bool lead = threadIdx.x == 0 && threadIdx.y < 3;   // three warps issue a share of the copies each
+    if (threadIdx.x == 0 && threadIdx.y == 0) {
+        for (int b = 0; b < NS; ++b) mbar_init(bars + b, 3);
         mbar_fence_init();
     }
     __syncthreads();
@@ -365,8 +363,7 @@ __device__ __forceinline__ void walk_tiles(unsigned char *smem, int gx, int run,
     auto issue = [&](int i) {
         if (!lead || i >= n) return;
         fence_proxy_async_smem();
-        mbar_expect_tx(bars + i % NS, TX);
-        load(xb, (r0 + i) * kTileH, smem + (i % NS) * STAGE, bars + i % NS);
+        load(threadIdx.y, xb, (r0 + i) * kTileH, smem + (i % NS) * STAGE, bars + i % NS);
     };
     pdl_wait();
     for (int i = 0; i < NS - 1; ++i) issue(i);
@@ -398,20 +395,23 @@ k_velocity_tiles(const __grid_constant__ VelArgs<float, float, SP> A, const __gr
     const int tx = threadIdx.x, ty = threadIdx.y, e0 = ty * kTileW + 4 * tx;
     QuadCoef<float, NM> C;
     uint2 key = make_uint2(0xffffffffu, 0xffffffffu);
-    auto load = [&](int xb, int zb, unsigned char *st, uint64_t *bar) {
-        tma_load_3d(st + L::o_sp, &M.p_halo, xb - 4, 0, zb - 3, bar);
-        tma_load_3d(st + L::o_sr, &M.rho_halo, xb, 0, zb, bar);
-        tma_load_3d(st + L::o_cls, &M.cls, xb, 0, zb, bar);
-        if (TS) tma_load_3d(st + L::o_kv, &M.kdt, xb, 0, zb, bar);
-#pragma unroll
-        for (int s = 0; s < 2; ++s) {
-            tma_load_3d(st + L::o_v + s * kTileN * 4, &M.v[2 * s], xb, 0, zb, bar);
-#pragma unroll
-            for (int m = 0; m < NM; ++m)
-                tma_load_3d(st + L::o_psi + (2 * m + s) * kTileN * sizeof(SP), &M.psi[m][2 * s], xb, 0, zb, bar);
+    auto load = [&](int w, int xb, int zb, unsigned char *st, uint64_t *bar) {
+        if (w == 0) {
+            mbar_expect_tx(bar, (unsigned)((L::SW * L::SH + L::RW * (kTileH + 1) + (TS ? kTileN : 0)) * 4 + kTileN * 2));
+            tma_load_3d(st + L::o_sp, &M.p_halo, xb - 4, 0, zb - 3, bar);
+            tma_load_3d(st + L::o_sr, &M.rho_halo, xb, 0, zb, bar);
+            tma_load_3d(st + L::o_cls, &M.cls, xb, 0, zb, bar);
+            if (TS) tma_load_3d(st + L::o_kv, &M.kdt, xb, 0, zb, bar);
+            return;
         }
+        const int s = w - 1;
+        mbar_expect_tx(bar, (unsigned)(kTileN * (4 + NM * sizeof(SP))));
+        tma_load_3d(st + L::o_v + s * kTileN * 4, &M.v[2 * s], xb, 0, zb, bar);
+#pragma unroll
+        for (int m = 0; m < NM; ++m)
+            tma_load_3d(st + L::o_psi + (2 * m + s) * kTileN * sizeof(SP), &M.psi[m][2 * s], xb, 0, zb, bar);
     };
-    walk_tiles<NS, L::stage, L::tx>(smem, gx, run, n_rows, A.mon, load, [&](int xb, int zb, unsigned char *st, auto wait) {
+    walk_tiles<NS, L::stage>(smem, gx, run, n_rows, A.mon, load, [&](int xb, int zb, unsigned char *st, auto wait) {
         PlanePos P;
         P.x0 = xb + 4 * tx;
         P.z = zb + ty;
@@ -489,18 +489,25 @@ k_pressure_tiles(const __grid_constant__ PresArgs<float, float, SP> A, const __g
     QuadCoef<float, NM> C;
     uint2 key = make_uint2(0xffffffffu, 0xffffffffu);
     PMax<float> pmax;
-    auto load = [&](int xb, int zb, unsigned char *st, uint64_t *bar) {
-        tma_load_3d(st + L::o_vx, TS ? &M.vx_ring : &M.vx_halo, xb - 4, 0, TS ? zb - 1 : zb, bar);
-        tma_load_3d(st + L::o_vz, TS ? &M.vz_ring : &M.vz_own, TS ? xb - 4 : xb, 0, zb - 4, bar);
-        tma_load_3d(st + L::o_p, &M.p_own, xb, 0, zb, bar);
-        tma_load_3d(st + L::o_kd, &M.kdt, xb, 0, zb, bar);
-        if (NL) tma_load_3d(st + L::o_bd, &M.b2dt, xb, 0, zb, bar);
-        if (TS) tma_load_3d(st + L::o_rh, &M.rho_own, xb, 0, zb, bar);
-        tma_load_3d(st + L::o_cls, &M.cls, xb, 0, zb, bar);
+    auto load = [&](int w, int xb, int zb, unsigned char *st, uint64_t *bar) {
+        if (w == 0) {
+            mbar_expect_tx(bar, (unsigned)((L::XW * L::XH + L::ZW * L::ZH) * 4));
+            tma_load_3d(st + L::o_vx, TS ? &M.vx_ring : &M.vx_halo, xb - 4, 0, TS ? zb - 1 : zb, bar);
+            tma_load_3d(st + L::o_vz, TS ? &M.vz_ring : &M.vz_own, TS ? xb - 4 : xb, 0, zb - 4, bar);
+        } else if (w == 1) {
+            mbar_expect_tx(bar, (unsigned)(kTileN * 4 * (2 + (NL ? 1 : 0) + (TS ? 1 : 0))));
+            tma_load_3d(st + L::o_p, &M.p_own, xb, 0, zb, bar);
+            tma_load_3d(st + L::o_kd, &M.kdt, xb, 0, zb, bar);
+            if (NL) tma_load_3d(st + L::o_bd, &M.b2dt, xb, 0, zb, bar);
+            if (TS) tma_load_3d(st + L::o_rh, &M.rho_own, xb, 0, zb, bar);
+        } else {
+            mbar_expect_tx(bar, (unsigned)(kTileN * (2 + NM * sizeof(SP))));
+            tma_load_3d(st + L::o_cls, &M.cls, xb, 0, zb, bar);
 #pragma unroll
-        for (int m = 0; m < NM; ++m) tma_load_3d(st + L::o_psi + m * kTileN * sizeof(SP), &M.psi[m], xb, 0, zb, bar);
+            for (int m = 0; m < NM; ++m) tma_load_3d(st + L::o_psi + m * kTileN * sizeof(SP), &M.psi[m], xb, 0, zb, bar);
+        }
     };
-    walk_tiles<NS, L::stage, L::tx>(smem, gx, run, n_rows, A.mon, load, [&](int xb, int zb, unsigned char *st, auto wait) {
+    walk_tiles<NS, L::stage>(smem, gx, run, n_rows, A.mon, load, [&](int xb, int zb, unsigned char *st, auto wait) {
         PlanePos P;
         P.x0 = xb + 4 * tx;
         P.z = zb + ty;
