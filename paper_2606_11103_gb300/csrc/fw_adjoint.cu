@@ -213,11 +213,12 @@ __global__ void __launch_bounds__(32 * kAdjRows, sizeof(R) == 4 ? 4 : 1) k_adj_p
         Io<R>::ld(A.fpsi2[m] + P.i, old[m]);
     }
     const bool in[3] = {adj_in_layer<R, DIM>(A, P, 0), adj_in_layer<R, DIM>(A, P, 1), adj_in_layer<R, DIM>(A, P, 2)};
-    R Q[4], gsp[4], stp[4], lst[4];
+    R Q[4], gsp[4], stp[4], lst[4], ik[4];
     CellCoef<R, NM> C;
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
         if (e == 0 || cls[e] != cls[e - 1]) C.load(A, cls[e], 2);
+        ik[e] = C.ik;
         const R r = in[0] || in[1] || in[2] ? adj_ramp(A, P, e) : R(1);
         lst[e] = -kd[e] * lp[e];
         const R rdiv = r * div[e], half = R(0.5) * lst[e];
@@ -245,13 +246,10 @@ __global__ void __launch_bounds__(32 * kAdjRows, sizeof(R) == 4 ? 4 : 1) k_adj_p
         R Qa[4] = {Q[0], Q[1], Q[2], Q[3]};
         if (in[ax]) {
             R a[4], b[4], lpn[4], po[4];
-            if (ax == 0) {
-                const R *pd = A.pdi[0] + P.c[0], *pa = A.pai[0] + P.c[0];
-                const R dq[4] = {pd[0], pd[1], pd[2], pd[3]}, aq[4] = {pa[0], pa[1], pa[2], pa[3]};
-                quad_layer_ab(A.lut, cls, 1, dq, aq, A.dt, a, b);
-            } else {
-                quad_layer_ab(A.lut, cls, 1, A.pdi[ax][P.c[ax]], A.pai[ax][P.c[ax]], A.dt, a, b);
-            }
+            if (ax == 0) quad_layer_ab(ik, A.pdi[0] + P.c[0], A.pai[0] + P.c[0], A.dt, a, b);
+            else if (A.pdi[ax][P.c[ax]] > R(0))
+                quad_layer_ab(ik, A.pdi[ax][P.c[ax]], A.pai[ax][P.c[ax]], A.dt, a, b);
+            else b[0] = b[1] = b[2] = b[3] = R(2);
             Io<R>::ld(A.L.lpsi2p[ax] + P.i, lpn);
             Io<R>::ld(A.fpsi2p[ax] + P.i, po);
 #pragma unroll
@@ -276,7 +274,7 @@ template <typename R, int DIM, int NM, int ax>
 __device__ __forceinline__ void adj_velocity_axis(const AdjArgs<R> &A, const AdjPos &P, const uint16_t (&cls)[4],
                                                   const R (&own)[4], const R (&rr)[4], R (&gs)[4])
 {
-    R lv[4], dq[4], g[4], nxt[4], ln[NM][4], old[NM][4], lg[4], lst[4];
+    R lv[4], dq[4], g[4], nxt[4], ln[NM][4], old[NM][4], lg[4], lst[4], ik[4];
     Io<R>::ld(A.L.lv[ax] + P.i, lv);
 #pragma unroll
     for (int m = 0; m < NM; ++m) {
@@ -297,6 +295,7 @@ __device__ __forceinline__ void adj_velocity_axis(const AdjArgs<R> &A, const Adj
         const bool live = P.c[0] + e < A.nx;
         if (ax == 0 ? P.c[0] + e + 1 >= A.nx : P.c[ax] + 1 >= P.n[ax]) nxt[e] = own[e];
         if (e == 0 || cls[e] != cls[e - 1]) C.load(A, cls[e], 1);
+        ik[e] = C.ik;
         lv[e] = live ? lv[e] - dq[e] : R(0);
         lst[e] = live ? div_face(-A.dt, fma(R(0.5), nxt[e], R(0.5) * own[e])) * lv[e] : R(0);
         const R rg = live ? rr[e] * g[e] : R(0), half = R(0.5) * lst[e];
@@ -315,13 +314,9 @@ __device__ __forceinline__ void adj_velocity_axis(const AdjArgs<R> &A, const Adj
     for (int m = 0; m < NM; ++m) Io<R>::st(A.L.lpsi1[m][ax] + P.i, ln[m]);
     if (adj_in_layer<R, DIM>(A, P, ax)) {
         R a[4], b[4], lpn[4];
-        if (ax == 0) {
-            const R *pd = A.pdh[0] + P.c[0], *pa = A.pah[0] + P.c[0];
-            const R d4[4] = {pd[0], pd[1], pd[2], pd[3]}, a4[4] = {pa[0], pa[1], pa[2], pa[3]};
-            quad_layer_ab(A.lut, cls, 0, d4, a4, A.dt, a, b);
-        } else {
-            quad_layer_ab(A.lut, cls, 0, A.pdh[ax][P.c[ax]], A.pah[ax][P.c[ax]], A.dt, a, b);
-        }
+        if (ax == 0) quad_layer_ab(ik, A.pdh[0] + P.c[0], A.pah[0] + P.c[0], A.dt, a, b);
+        else if (A.pdh[ax][P.c[ax]] > R(0)) quad_layer_ab(ik, A.pdh[ax][P.c[ax]], A.pah[ax][P.c[ax]], A.dt, a, b);
+        else b[0] = b[1] = b[2] = b[3] = R(2);
         Io<R>::ld(A.L.lpsi1p[ax] + P.i, lpn);
 #pragma unroll
         for (int e = 0; e < 4; ++e) {

@@ -65,19 +65,22 @@ __device__ __forceinline__ void plane_ramp(const Geo<R> &G, const PlanePos &P, R
     for (int e = 0; e < 4; ++e) rr[e] = ramp_of(fmax(layer_depth<R>(P.x0 + e, G.nx, G.wabs), sz), inv_lr);
 }
 
-// Coefficients of the absorbing mechanism along ax (0 or 2) of the quad
+// The absorbing mechanism along ax (0 or 2) of the quad: ik its cells'
+// 1 / kappa, g the derivative, pp the memory; its term is added to st
 template <typename R>
-__device__ __forceinline__ void plane_layer_ab(const R *const (&pd)[3], const R *const (&pa)[3], const R *lut,
-                                               const uint16_t (&cls)[4], int offK, R dt, int ax, const PlanePos &P,
-                                               R (&a)[4], R (&b)[4])
+__device__ __forceinline__ void plane_layer(const R *const (&pd)[3], const R *const (&pa)[3], const R (&ik)[4], R dt,
+                                            int ax, const PlanePos &P, const R (&g)[4], R (&pp)[4], R (&st)[4])
 {
+    R a[4], b[4], w[4] = {R(0.5), R(0.5), R(0.5), R(0.5)};
     if (ax == 0) {
-        const R *d = pd[0] + P.x0, *al = pa[0] + P.x0;
-        const R dq[4] = {d[0], d[1], d[2], d[3]}, aq[4] = {al[0], al[1], al[2], al[3]};
-        quad_layer_ab(lut, cls, offK, dq, aq, dt, a, b);
+        quad_layer_ab(ik, pd[0] + P.x0, pa[0] + P.x0, dt, a, b);
+        quad_layer_weights(b, w);
     } else {
-        quad_layer_ab(lut, cls, offK, pd[2][P.z], pa[2][P.z], dt, a, b);
+        const R d = pd[2][P.z];
+        if (!(d > R(0))) return;
+        quad_layer_ab(ik, d, pa[2][P.z], dt, a, b);
     }
+    quad_layer(a, b, w, g, pp, st);
 }
 
 // Time-space stencil (see vel_gradient_ts): gradient of p at the two faces of
@@ -220,10 +223,9 @@ k_velocity_plane(const __grid_constant__ VelArgs<R, SS, SP> A, int gx)
         R(&v)[4] = vv[ax / 2], (&pa)[NM][4] = ps[ax / 2], stv[4];
         quad_stretch<R, NM>(C, g[ax], rr, G.hs1, pa, stv);
         if (in[ax]) {
-            R pp[4], a[4], b[4];
+            R pp[4];
             Io<SS>::ld(A.psip[ax] + row, pp);
-            plane_layer_ab(A.pd, A.pa, A.lut, cls4, 0, G.dt, ax, P, a, b);
-            quad_layer(a, b, g[ax], pp, stv);
+            plane_layer(A.pd, A.pa, C.ik, G.dt, ax, P, g[ax], pp, stv);
             Io<SS>::st(wr_at(A.psip[ax] + row, A.wofs), pp);
         }
 #pragma unroll
@@ -291,10 +293,9 @@ k_pressure_plane(const __grid_constant__ PresArgs<R, SS, SP> A, int gx)
 #pragma unroll
         for (int ax = 0; ax < 3; ax += 2) {
             if (!in[ax]) continue;
-            R pp[4], a[4], b[4];
+            R pp[4];
             Io<SS>::ld(A.psip[ax] + row, pp);
-            plane_layer_ab(A.pd, A.pa, A.lut, cls4, 1, G.dt, ax, P, a, b);
-            quad_layer(a, b, qd[ax], pp, stp);
+            plane_layer(A.pd, A.pa, C.ik, G.dt, ax, P, qd[ax], pp, stp);
             Io<SS>::st(wr_at(A.psip[ax] + row, A.wofs), pp);
         }
 #pragma unroll
@@ -463,9 +464,7 @@ k_velocity_tiles(const __grid_constant__ VelArgs<float, float, SP> A, const __gr
                 Sm<SP>::ld(reinterpret_cast<const SP *>(st + L::o_psi) + (2 * m + ax / 2) * kTileN + e0, ps[m]);
             quad_stretch<float, NM>(C, g[ax], rr, G.hs1, ps, stv);
             if (in[ax]) {
-                float a[4], b[4];
-                plane_layer_ab(A.pd, A.pa, A.lut, cls4, 0, G.dt, ax, P, a, b);
-                quad_layer(a, b, g[ax], pp[ax], stv);
+                plane_layer(A.pd, A.pa, C.ik, G.dt, ax, P, g[ax], pp[ax], stv);
                 Io<float>::st(A.psip[ax] + P.row, pp[ax]);
             }
 #pragma unroll
@@ -561,9 +560,7 @@ k_pressure_tiles(const __grid_constant__ PresArgs<float, float, SP> A, const __g
 #pragma unroll
         for (int ax = 0; ax < 3; ax += 2) {
             if (!in[ax]) continue;
-            float a[4], b[4];
-            plane_layer_ab(A.pd, A.pa, A.lut, cls4, 1, G.dt, ax, P, a, b);
-            quad_layer(a, b, qd[ax], pp[ax], stp);
+            plane_layer(A.pd, A.pa, C.ik, G.dt, ax, P, qd[ax], pp[ax], stp);
             Io<float>::st(A.psip[ax] + P.row, pp[ax]);
         }
 #pragma unroll
