@@ -667,21 +667,44 @@ std::vector<long long> mask_to_index(const fw_medium *m, const uint8_t *mask)
     return out;
 }
 
-int choose_zseg(const fw_medium *m)
+// Depth planes per CTA of a 3D sweep with `tiles` CTAs per depth segment: the
+// length with the earliest last CTA when the segments are handed to the
+// device's slots in order, a CTA costing its planes plus half a plane of
+// start-up; the last, shorter segment fills up a wave.  8 to 24 planes where
+// the grid is only a few waves of CTAs, else 8 to 14, where the estimate
+// matters little and more CTAs balance better.  Measured, 128^3, N = 4 (32
+// tiles; 304 and 456 slots): velocity 8 / 14 / 16 planes 53.7 / 52.0 / 55.1 us,
+// pressure 8 / 9 / 10 / 16 planes 38 / 31.1 / 34.7 / 39.2 us; 384^3, binary16,
+// 10 / 16 / 24 planes 745 / 763 / 778 and 399 / 400 / 404 us; 512^3 8 to 24
+// planes alike within 0.7 %.
+int choose_zseg(long long tiles, int nz, int slots)
 {
     // tuning override: FWGB_ZSEG planes per CTA (8..1024)
     if (const char *e = std::getenv("FWGB_ZSEG")) {
         int z = std::atoi(e);
         if (z >= 8 && z <= 1024) return z;
     }
-    // 16 planes per CTA measured best on the 512^3 workload (L2 sharing of
-    // the halo planes between concurrently resident CTAs); at least 8 waves
-    // of CTAs over the 152 SMs
-    const int tw = m->es == 8 ? 64 : 128, by = 8;
-    long long tiles = (long long)((m->NX + tw - 1) / tw) * ((m->NY + by - 1) / by);
-    int z = 16;
-    while (z > 8 && tiles * ((m->NZ + z - 1) / z) < 152LL * 8) z /= 2;
-    return z;
+    if (slots < 1) return 16;
+    const int longest = tiles * ((nz + 15) / 16) >= 4LL * slots ? 14 : 24;
+    int best = 16;
+    double best_end = 1e30;
+    for (int z = 8; z <= longest; ++z) {
+        const double full = z + 0.5, rem = nz % z + 0.5;          // planes of a CTA, of one of the last segment
+        const long long n_full = tiles * (nz / z), n_rem = nz % z ? tiles : 0, waves = n_full / slots,
+                        extra = n_full % slots, idle = slots - extra;
+        double end = waves * full + (extra ? full : 0.0);
+        if (n_rem) {   // on the slots without an extra full CTA alone, or the rest of them on all after that
+            const long long fit = idle * (long long)(full / rem), over = std::max(0LL, n_rem - fit);
+            const double alone = waves * full + rem * ((n_rem + idle - 1) / idle);
+            const double after = (waves + 1) * full + rem * ((over + slots - 1) / slots);
+            end = std::max(end, over ? std::min(alone, after) : alone);
+        }
+        if (end < best_end) {
+            best_end = end;
+            best = z;
+        }
+    }
+    return best;
 }
 
 int create_common(const fw_grid *g, const float *c, const float *rho, const float *beta,
@@ -758,7 +781,6 @@ int create_common(const fw_grid *g, const float *c, const float *rho, const floa
     m->cls = static_cast<uint16_t *>(at(L.cls));
     m->lut = at(L.lut);
     m->cdev = at(L.cdev);
-    m->zseg = choose_zseg(m);
     setup_tma(m);
     // maps into the padded layout with inheritance
     if (d.es == 8) {
@@ -839,6 +861,10 @@ int create_common(const fw_grid *g, const float *c, const float *rho, const floa
     }
     if (cudaStreamCreateWithFlags(&m->cap_stream, cudaStreamNonBlocking) != cudaSuccess) { release(m); return FW_ERR_CUDA; }
     if (launch_sweep(m, s, 4) != cudaSuccess) { release(m); return FW_ERR_CUDA; }
+    if (m->ndim == 3) {
+        const long long tiles = ((m->NX + 63LL) / 64) * (m->es == 8 ? (m->NY + 3LL) / 4 : (m->NY + 7LL) / 8);
+        for (int i = 0; i < 2; ++i) m->zseg[i] = choose_zseg(tiles, m->NZ, m->slots[i]);
+    }
     if (cudaStreamSynchronize(s) != cudaSuccess) { release(m); return FW_ERR_CUDA; }
     noalloc_prepare();
     m->last_stream = s;

@@ -123,7 +123,8 @@ struct fw_medium {
     cudaStream_t last_stream = nullptr;
     cudaStream_t cap_stream = nullptr;
     std::map<int, fwgb::Graph> graphs;
-    int zseg = 32;
+    int zseg[2] = {16, 16};          // depth planes per CTA of the 3D velocity and pressure sweeps
+    mutable int slots[2] = {0, 0};   // CTAs of either that the device holds at once, found at creation
     double psi_pref = 10.0;          // pressure reference [Pa] of binary16 memory variables
     int time_order = 2;              // 2: leapfrog; 4: time-space stencil (Sec. 3.3)
     double ts_a[4][4] = {};          // time-space weights a_m = sum_n ts_a[m][n] r^(2n)

@@ -49,7 +49,6 @@ template <typename R> Geo<R> make_geo(const fw_medium *m)
     g.nz = m->NZ;
     g.px = m->px;
     g.plane = (long long)m->plane;
-    g.zseg = m->zseg;
     g.wabs = m->wabs;
     // 8th-order staggered weights (Taylor) divided by dx
     const double cm[4] = {1225.0 / 1024.0, -245.0 / 3072.0, 49.0 / 5120.0, -5.0 / 7168.0};
@@ -182,6 +181,7 @@ VelArgs<R, SS, SP> vel_args(const fw_medium *m, const StepImages *im)
     VelArgs<R, SS, SP> va{};
     va.g = make_geo<R>(m);
     va.p = static_cast<const SS *>(at.rd(m->p));
+    va.g.zseg = m->zseg[0];
     va.wofs = im ? im->wofs : 0;
     for (int ax = 0; ax < 3; ++ax) {
         va.v[ax] = static_cast<SS *>(at.rd(m->v[ax]));
@@ -205,6 +205,7 @@ PresArgs<R, SS, SP> pres_args(const fw_medium *m, const StepImages *im)
     PresArgs<R, SS, SP> pa{};
     pa.g = make_geo<R>(m);
     pa.p = static_cast<SS *>(at.rd(m->p));
+    pa.g.zseg = m->zseg[1];
     pa.wofs = im ? im->wofs : 0;
     for (int ax = 0; ax < 3; ++ax) {
         pa.v[ax] = static_cast<const SS *>(at.nw(m->v[ax]));   // this step's velocity
@@ -300,6 +301,13 @@ cudaError_t launch_3d_as(const fw_medium *m, cudaStream_t s, int which, const St
         cudaError_t e = cudaFuncSetAttribute(kv, attr, (int)LV::bytes);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(kp, attr, (int)LP::bytes);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(kpn, attr, (int)LP::bytes);
+        int per_sm[2] = {0, 0}, dev = 0, sms = 0;
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm[0], kv, BX * BYV, LV::bytes);
+        if (e == cudaSuccess)
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm[1], m->nonlinear ? kpn : kp, BX * BYP, LP::bytes);
+        if (e == cudaSuccess) e = cudaGetDevice(&dev);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        for (int i = 0; i < 2; ++i) m->slots[i] = per_sm[i] * sms;
         return e;
     }
     MapsArg<TMA, VelMaps> vm;
@@ -308,14 +316,15 @@ cudaError_t launch_3d_as(const fw_medium *m, cudaStream_t s, int which, const St
         vm = m->vel_maps;
         pm = m->pres_maps;
     }
-    const int gx = (m->NX + 4 * BX - 1) / (4 * BX), gz = (m->NZ + m->zseg - 1) / m->zseg;
+    const int gx = (m->NX + 4 * BX - 1) / (4 * BX);
+    auto segs = [m](int i) { return (m->NZ + m->zseg[i] - 1) / m->zseg[i]; };
     const bool pdl = !(which & 8);
     cudaError_t e = cudaSuccess;
     if (which & 1)
-        e = launch_kernel(kv, dim3(gx, (m->NY + BYV - 1) / BYV, gz), dim3(BX, BYV), LV::bytes, s, pdl,
+        e = launch_kernel(kv, dim3(gx, (m->NY + BYV - 1) / BYV, segs(0)), dim3(BX, BYV), LV::bytes, s, pdl,
                           vel_args<R, SS, SP, NM>(m, im), vm);
     if (e == cudaSuccess && (which & 2))
-        e = launch_kernel(m->nonlinear ? kpn : kp, dim3(gx, (m->NY + BYP - 1) / BYP, gz), dim3(BX, BYP), LP::bytes, s,
+        e = launch_kernel(m->nonlinear ? kpn : kp, dim3(gx, (m->NY + BYP - 1) / BYP, segs(1)), dim3(BX, BYP), LP::bytes, s,
                           pdl, pres_args<R, SS, SP, NM>(m, im), pm);
     return e;
 }
@@ -327,12 +336,11 @@ template <typename R, typename SS, typename SP, int NM, bool TS>
 cudaError_t launch_3d(const fw_medium *m, cudaStream_t s, int which, const StepImages *im)
 {
     if constexpr (sizeof(R) == 4) {
-        if (which & 4) {
-            const cudaError_t e = launch_3d_as<R, SS, SP, NM, TS, true>(m, s, which, im);
-            if (e != cudaSuccess) return e;
-        } else if (m->tma && !im) {
-            return launch_3d_as<R, SS, SP, NM, TS, true>(m, s, which, im);
+        if (which & 4) {   // both forms: image steps take the second one
+            const cudaError_t e = launch_3d_as<R, SS, SP, NM, TS, false>(m, s, which, im);
+            return e == cudaSuccess && m->tma ? launch_3d_as<R, SS, SP, NM, TS, true>(m, s, which, im) : e;
         }
+        if (m->tma && !im) return launch_3d_as<R, SS, SP, NM, TS, true>(m, s, which, im);
     }
     return launch_3d_as<R, SS, SP, NM, TS, false>(m, s, which, im);
 }
