@@ -273,9 +273,9 @@ int fw_run(fw_medium *m, int n_steps, void *stream);
 
 /* fw_step with a CUDA event around each sweep: advances n_steps on stream
  * (plain launches), waits for them, and returns the summed device time [ms]
- * of the velocity sweeps, the pressure sweeps and the source/receiver
- * kernels, the device time from the first launch to the last, and the number
- * of kernels launched.  Output pointers may be NULL.  For measurement;
+ * of the velocity sweeps and of the pressure sweeps (which inject the sources
+ * and record the receivers, so *ms_io is 0), the device time from the first
+ * launch to the last, and the number of kernels launched.  Output pointers may be NULL.  For measurement;
  * results equal fw_step's. */
 int fw_step_timed(fw_medium *m, int n_steps, void *stream, double *ms_velocity, double *ms_pressure,
                   double *ms_io, double *ms_total, int *n_launches);

@@ -41,8 +41,10 @@ namespace fwgb {
 void *device_alloc(size_t bytes);
 void device_free(void *p);
 size_t state_image_bytes(const fw_medium *m);
-cudaError_t image_step_f32(const fw_medium *m, const StepImages &im, const int *zero, int it, bool pdl, cudaStream_t s);
-cudaError_t image_step_f64(const fw_medium *m, const StepImages &im, const int *zero, int it, bool pdl, cudaStream_t s);
+cudaError_t image_step_f32(const fw_medium *m, const StepImages &im, const int *zero, int it, bool record, bool pdl,
+                           cudaStream_t s);
+cudaError_t image_step_f64(const fw_medium *m, const StepImages &im, const int *zero, int it, bool record, bool pdl,
+                           cudaStream_t s);
 }  // namespace fwgb
 
 using namespace fwgb;
@@ -660,8 +662,8 @@ int gradient_impl(fw_medium *m, int n_steps, int K, const void *G, const void *a
             char *wr = segs[si & 1] + (size_t)(k - k0) * SB;
             const StepImages im{rd, (long long)(wr - rd)};
             const int itk = (int)(it0 + k);
-            if ((sizeof(R) == 8 ? image_step_f64(m, im, static_cast<const int *>(zero.p), itk, k > k0, ss.side)
-                                : image_step_f32(m, im, static_cast<const int *>(zero.p), itk, k > k0, ss.side)) != cudaSuccess)
+            if ((sizeof(R) == 8 ? image_step_f64(m, im, static_cast<const int *>(zero.p), itk, false, k > k0, ss.side)
+                                : image_step_f32(m, im, static_cast<const int *>(zero.p), itk, false, k > k0, ss.side)) != cudaSuccess)
                 return FW_ERR_CUDA;
             rd = wr;
         }

@@ -15,12 +15,10 @@
 #include <vector>
 
 namespace fwgb {
-cudaError_t sweeps_f32(const fw_medium *m, cudaStream_t s, int which);
-cudaError_t sweeps_bf16(const fw_medium *m, cudaStream_t s, int which);
-cudaError_t sweeps_f16(const fw_medium *m, cudaStream_t s, int which);
-cudaError_t sweeps_f64(const fw_medium *m, cudaStream_t s, int which);
-cudaError_t io_f32(const fw_medium *m, int j, bool pdl, cudaStream_t s);
-cudaError_t io_f64(const fw_medium *m, int j, bool pdl, cudaStream_t s);
+cudaError_t sweeps_f32(const fw_medium *m, cudaStream_t s, int which, int j);
+cudaError_t sweeps_bf16(const fw_medium *m, cudaStream_t s, int which, int j);
+cudaError_t sweeps_f16(const fw_medium *m, cudaStream_t s, int which, int j);
+cudaError_t sweeps_f64(const fw_medium *m, cudaStream_t s, int which, int j);
 cudaError_t launch_advance(int *d_it, int n, bool pdl, cudaStream_t s);
 void noalloc_prepare();
 using EncodeTiledFn = CUresult (*)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
@@ -41,7 +39,7 @@ using namespace fwgb;
 
 namespace {
 
-cudaError_t launch_sweep(const fw_medium *m, cudaStream_t s, int which);
+cudaError_t launch_sweep(const fw_medium *m, cudaStream_t s, int which, int j = 0);
 
 // ---- allocator --------------------------------------------------------------
 std::mutex g_alloc_mu;
@@ -346,7 +344,7 @@ struct Layout {
     size_t off_state_end = 0;   // [0, off_state_end): state + counters (checkpoint image)
     size_t total = 0;
     size_t p, v[3], psi1[FW_MAX_MECH][3], psi2[FW_MAX_MECH], psi1p[3], psi2p[3], it, mon;
-    size_t kdt, rho, b2dt, cls, lut, cdev, prof[3][4];
+    size_t kdt, rho, b2dt, cls, lut, cdev, prof[3][4], io_off;
 };
 
 struct Dims {
@@ -357,6 +355,18 @@ struct Dims {
 
 int axis_len(const Dims &d, int ax) { return ax == 0 ? d.NX : (ax == 1 ? d.NY : d.NZ); }
 bool axis_on(const Dims &d, int ax) { return !(d.ndim == 2 && ax == 1); }
+
+// tiles of the pressure sweep (fw_launch.cuh: Tile3 and the 2D tiles)
+IoTiling io_tiling(int ndim, int nx, int ny, int nz, int es)
+{
+    IoTiling t{};
+    t.w = ndim == 3 ? 64 : 128;
+    t.h = ndim == 3 && es == 4 ? 8 : 4;
+    t.gx = (nx + t.w - 1) / t.w;
+    t.gy = ((ndim == 3 ? ny : nz) + t.h - 1) / t.h;
+    t.n = (long long)t.gx * t.gy * (ndim == 3 ? nz : 1);
+    return t;
+}
 
 Layout make_layout(const Dims &d, int n_classes)
 {
@@ -388,6 +398,7 @@ Layout make_layout(const Dims &d, int n_classes)
     L.lut = take((size_t)std::max(n_classes, 1) * kLutStride * d.es);
     for (int ax = 0; ax < 3; ++ax)
         for (int k = 0; k < 4; ++k) L.prof[ax][k] = take((size_t)axis_len(d, ax) * d.es + 64);
+    L.io_off = take((io_tiling(d.ndim, d.NX, d.NY, d.NZ, d.es).n + 1) * sizeof(int));
     L.total = o;
     return L;
 }
@@ -558,35 +569,24 @@ void release(fw_medium *m)
     if (m->cap_stream) cudaStreamDestroy(m->cap_stream);
     dev_free(m->src_buf);
     dev_free(m->rcv_buf);
+    dev_free(m->ent_buf);
     dev_free(m->slab);
     delete m;
 }
 
-cudaError_t launch_sweep(const fw_medium *m, cudaStream_t s, int which)
+cudaError_t launch_sweep(const fw_medium *m, cudaStream_t s, int which, int j)
 {
     switch (m->storage) {
-    case FW_STORE_F32: return sweeps_f32(m, s, which);
-    case FW_STORE_BF16: return sweeps_bf16(m, s, which);
-    case FW_STORE_F16: return sweeps_f16(m, s, which);
-    default: return sweeps_f64(m, s, which);
+    case FW_STORE_F32: return sweeps_f32(m, s, which, j);
+    case FW_STORE_BF16: return sweeps_bf16(m, s, which, j);
+    case FW_STORE_F16: return sweeps_f16(m, s, which, j);
+    default: return sweeps_f64(m, s, which, j);
     }
-}
-
-cudaError_t launch_io_any(const fw_medium *m, int j, bool pdl, cudaStream_t s)
-{
-    return m->storage == FW_STORE_F64 ? io_f64(m, j, pdl, s) : io_f32(m, j, pdl, s);
-}
-
-cudaError_t launch_step(const fw_medium *m, int j, cudaStream_t s)
-{
-    cudaError_t e = launch_sweep(m, s, 3);
-    if (e != cudaSuccess) return e;
-    return launch_io_any(m, j, true, s);
 }
 
 int enqueue_steps(fw_medium *m, int n, cudaStream_t s)
 {
-    for (int j = 0; j < n; ++j) FW_CK(launch_step(m, j, s));
+    for (int j = 0; j < n; ++j) FW_CK(launch_sweep(m, s, 3, j));
     FW_CK(launch_advance(m->d_it, n, true, s));
     return FW_OK;
 }
@@ -781,6 +781,7 @@ int create_common(const fw_grid *g, const float *c, const float *rho, const floa
     m->cls = static_cast<uint16_t *>(at(L.cls));
     m->lut = at(L.lut);
     m->cdev = at(L.cdev);
+    m->io_off = static_cast<int *>(at(L.io_off));
     setup_tma(m);
     // maps into the padded layout with inheritance
     if (d.es == 8) {
@@ -1052,26 +1053,64 @@ int fw_create_medium(const fw_grid *g, const float *c, const float *rho, const f
     return create_common(g, c, rho, beta, idx.data(), classes, storage, (cudaStream_t)stream, out);
 }
 
-// Source/receiver pairs on one cell: the combined injection-and-recording
-// kernel lets the source's thread record the receiver there (after the
-// injection), so no two threads touch one cell.  Both lists are sorted.
+// The lists behind injection and recording, from the sorted cells of the
+// sources and of the receivers: which receiver shares a source's cell and the
+// reverse (the adjoint's kernel lets one thread handle such a cell), and the
+// pressure sweep's entries, one per cell, ordered by tile.  A list no longer
+// than the last one needs no device memory, so after a set has been dropped
+// this cannot fail for want of it.
 static int upload_io_map(fw_medium *m, cudaStream_t s)
 {
     const std::vector<long long> &a = m->h_src_idx, &b = m->h_rcv_idx;
     std::vector<int> sr(a.size(), -1), rs(b.size(), -1);
-    for (size_t i = 0, j = 0; i < a.size() && j < b.size();) {
-        if (a[i] < b[j]) ++i;
-        else if (b[j] < a[i]) ++j;
-        else {
+    std::vector<IoEntry> e;
+    e.reserve(a.size() + b.size());
+    for (size_t i = 0, j = 0; i < a.size() || j < b.size();) {
+        if (j == b.size() || (i < a.size() && a[i] < b[j])) {
+            e.push_back({a[i], (int)i, -1});
+            ++i;
+        } else if (i == a.size() || b[j] < a[i]) {
+            e.push_back({b[j], -1, (int)j});
+            ++j;
+        } else {
             sr[i] = (int)j;
             rs[j] = (int)i;
+            e.push_back({a[i], (int)i, (int)j});
             ++i;
             ++j;
         }
     }
+    // counting sort by tile
+    const IoTiling T = io_tiling(m->ndim, m->NX, m->NY, m->NZ, m->es);
+    auto tile = [&](long long cell) {
+        const long long r = cell / m->px, x = cell % m->px, y = r % m->NY, z = r / m->NY;
+        return m->ndim == 3 ? (y / T.h * T.gx + x / T.w) * m->NZ + z : z / T.h * T.gx + x / T.w;
+    };
+    std::vector<int> off;
+    std::vector<IoEntry> sorted(e.size());
+    if (!e.empty()) {
+        off.assign((size_t)T.n + 1, 0);
+        for (const IoEntry &x : e) ++off[(size_t)tile(x.cell) + 1];
+        for (size_t i = 0; i < (size_t)T.n; ++i) off[i + 1] += off[i];
+        std::vector<int> at(off.begin(), off.end() - 1);
+        for (const IoEntry &x : e) sorted[(size_t)at[(size_t)tile(x.cell)]++] = x;
+        if (m->ent_cap < e.size()) {
+            void *nb = dev_alloc(e.size() * sizeof(IoEntry));
+            if (!nb) return FW_ERR_NOMEM;
+            dev_free(m->ent_buf);
+            m->ent_buf = nb;
+            m->ent_cap = e.size();
+        }
+    }
+    m->n_ent = 0;                  // no entries should a copy fail
     if (m->src_rcv && !sr.empty()) FW_CK(cudaMemcpyAsync(m->src_rcv, sr.data(), sr.size() * 4, cudaMemcpyHostToDevice, s));
     if (m->rcv_src && !rs.empty()) FW_CK(cudaMemcpyAsync(m->rcv_src, rs.data(), rs.size() * 4, cudaMemcpyHostToDevice, s));
+    if (!e.empty()) {
+        FW_CK(cudaMemcpyAsync(m->io_off, off.data(), off.size() * 4, cudaMemcpyHostToDevice, s));
+        FW_CK(cudaMemcpyAsync(m->ent_buf, sorted.data(), sorted.size() * sizeof(IoEntry), cudaMemcpyHostToDevice, s));
+    }
     FW_CK(cudaStreamSynchronize(s));
+    m->n_ent = (int)e.size();
     return FW_OK;
 }
 
@@ -1135,7 +1174,12 @@ int fw_set_sources(fw_medium *m, const uint8_t *mask, const float *waveforms, in
     m->n_wave = n_wave;
     m->wave_len = n_steps;
     m->h_src_idx = std::move(idx);
-    if (int rc = upload_io_map(m, s)) return rc;
+    if (int rc = upload_io_map(m, s)) {
+        m->n_src = 0;                  // no sources; the receivers' entries as they were
+        m->h_src_idx.clear();
+        upload_io_map(m, s);
+        return rc;
+    }
     if (m->storage == FW_STORE_F16) return set_psi_reference(m, waveforms, wl);
     return FW_OK;
 }
@@ -1174,7 +1218,13 @@ int fw_set_receivers(fw_medium *m, const uint8_t *mask, int decim, int n_steps)
     m->n_rec = nrec;
     m->decim = decim;
     m->h_rcv_idx = std::move(idx);
-    return upload_io_map(m, s);
+    const int rc = upload_io_map(m, s);
+    if (rc) {
+        m->n_rcv = m->n_rec = 0;       // no receivers; the sources' entries as they were
+        m->h_rcv_idx.clear();
+        upload_io_map(m, s);
+    }
+    return rc;
 }
 
 int fw_step(fw_medium *m, int n_steps, void *stream)
@@ -1230,44 +1280,38 @@ int fw_step_timed(fw_medium *m, int n_steps, void *stream, double *ms_velocity, 
     cudaStream_t s = (cudaStream_t)stream;
     // all events exist before the first is recorded, so host-side creation
     // never shows up as device time
-    std::vector<cudaEvent_t> ev(3 * (size_t)n_steps + 1, nullptr);
+    std::vector<cudaEvent_t> ev(2 * (size_t)n_steps + 2, nullptr);
     for (auto &e : ev)
         if (cudaEventCreate(&e) != cudaSuccess) {
             for (auto &x : ev) if (x) cudaEventDestroy(x);
             return FW_ERR_CUDA;
         }
     int rc = FW_OK;
-    int launches = 0;
-    for (int j = 0; j < n_steps && rc == FW_OK; ++j) {
-        if (cudaEventRecord(ev[3 * j], s) != cudaSuccess || launch_sweep(m, s, 1 | 8) != cudaSuccess ||
-            cudaEventRecord(ev[3 * j + 1], s) != cudaSuccess || launch_sweep(m, s, 2 | 8) != cudaSuccess ||
-            cudaEventRecord(ev[3 * j + 2], s) != cudaSuccess || launch_io_any(m, j, false, s) != cudaSuccess)
+    const size_t last = 2 * (size_t)n_steps;
+    for (int j = 0; j < n_steps && rc == FW_OK; ++j)
+        if (cudaEventRecord(ev[2 * j], s) != cudaSuccess || launch_sweep(m, s, 1 | 8, j) != cudaSuccess ||
+            cudaEventRecord(ev[2 * j + 1], s) != cudaSuccess || launch_sweep(m, s, 2 | 8, j) != cudaSuccess)
             rc = FW_ERR_CUDA;
-        launches += 2 + (m->n_src + m->n_rcv > 0);
-    }
-    if (rc == FW_OK) {
-        launches += 1;
-        if (launch_advance(m->d_it, n_steps, false, s) != cudaSuccess || cudaEventRecord(ev[3 * (size_t)n_steps], s) != cudaSuccess ||
-            cudaEventSynchronize(ev[3 * (size_t)n_steps]) != cudaSuccess)
-            rc = FW_ERR_CUDA;
-    }
-    double tv = 0, tp = 0, ti = 0;
+    if (rc == FW_OK &&
+        (cudaEventRecord(ev[last], s) != cudaSuccess || launch_advance(m->d_it, n_steps, false, s) != cudaSuccess ||
+         cudaEventRecord(ev[last + 1], s) != cudaSuccess || cudaEventSynchronize(ev[last + 1]) != cudaSuccess))
+        rc = FW_ERR_CUDA;
+    double tv = 0, tp = 0;
     float tot = 0;
     for (int j = 0; j < n_steps && rc == FW_OK; ++j) {
-        float a = 0, b = 0, c = 0;
-        cudaEventElapsedTime(&a, ev[3 * j], ev[3 * j + 1]);
-        cudaEventElapsedTime(&b, ev[3 * j + 1], ev[3 * j + 2]);
-        cudaEventElapsedTime(&c, ev[3 * j + 2], ev[3 * j + 3]);
-        tv += a; tp += b; ti += c;
+        float a = 0, b = 0;
+        cudaEventElapsedTime(&a, ev[2 * j], ev[2 * j + 1]);
+        cudaEventElapsedTime(&b, ev[2 * j + 1], ev[2 * j + 2]);
+        tv += a; tp += b;
     }
-    if (rc == FW_OK && n_steps > 0) cudaEventElapsedTime(&tot, ev[0], ev[3 * (size_t)n_steps]);
+    if (rc == FW_OK && n_steps > 0) cudaEventElapsedTime(&tot, ev[0], ev[last + 1]);
     for (auto &e : ev) cudaEventDestroy(e);
     if (rc) return rc;
     if (ms_velocity) *ms_velocity = tv;
     if (ms_pressure) *ms_pressure = tp;
-    if (ms_io) *ms_io = ti;
+    if (ms_io) *ms_io = 0.0;
     if (ms_total) *ms_total = tot;
-    if (n_launches) *n_launches = launches;
+    if (n_launches) *n_launches = 2 * n_steps + 1;
     m->step += n_steps;
     m->last_stream = s;
     return FW_OK;

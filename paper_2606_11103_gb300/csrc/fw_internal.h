@@ -70,6 +70,22 @@ struct StepImages {
     long long wofs;
 };
 
+// A cell that holds a source, a receiver or both: its index in the padded
+// layout and the source's and receiver's numbers (-1: none)
+struct IoEntry {
+    long long cell;
+    int src, rcv;
+};
+
+// Tiles of the pressure sweep's CTAs by kernel axes, in 3D one per depth plane,
+// the planes of a tile following each other; the entries of a medium's cells
+// are ordered by tile
+struct IoTiling {
+    int w, h;            // columns, and rows of y (3D) or depth (2D)
+    int gx, gy;          // tiles along x, and along y (3D) or depth (2D)
+    long long n;         // number of tiles
+};
+
 struct Graph {
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
@@ -112,6 +128,12 @@ struct fw_medium {
     int *wave_of = nullptr;
     int n_src = 0, n_wave = 0, wave_len = 0;
     int n_rcv = 0, n_rec = 0, decim = 1;
+    // the cells with a source or a receiver, ordered by tile, and where each
+    // tile's entries begin (io_off: io_tiling(m).n + 1 values, in the slab)
+    void *ent_buf = nullptr;
+    size_t ent_cap = 0;
+    int n_ent = 0;
+    int *io_off = nullptr;
     // cells that hold both a source and a receiver: per source the receiver
     // there (or -1), per receiver the source there (or -1); host copies of
     // both index lists to rebuild them

@@ -2,11 +2,14 @@
 #include "fw_launch.cuh"
 
 namespace fwgb {
-cudaError_t sweeps_f32(const fw_medium *m, cudaStream_t s, int which) { return launch_sweeps<float, float, float>(m, s, which); }
-cudaError_t io_f32(const fw_medium *m, int j, bool pdl, cudaStream_t s) { return launch_io<float, float>(m, j, pdl, s); }
-cudaError_t image_step_f32(const fw_medium *m, const StepImages &im, const int *zero, int it, bool pdl, cudaStream_t s)
+cudaError_t sweeps_f32(const fw_medium *m, cudaStream_t s, int which, int j)
 {
-    return launch_image_step<float, float>(m, im, zero, it, pdl, s);
+    return launch_step_sweeps<float, float, float>(m, s, which, j);
+}
+cudaError_t image_step_f32(const fw_medium *m, const StepImages &im, const int *zero, int it, bool record, bool pdl,
+                           cudaStream_t s)
+{
+    return launch_image_step<float, float>(m, im, zero, it, record, pdl, s);
 }
 __global__ void k_advance(int *d_it, int n)
 {

@@ -198,8 +198,16 @@ VelArgs<R, SS, SP> vel_args(const fw_medium *m, const StepImages *im)
     return va;
 }
 
+// which step of the medium a pressure sweep injects and records: *d_it + j
+// (its own counter); image steps give theirs
+struct StepIo {
+    const int *d_it;
+    int j;
+    bool record;
+};
+
 template <typename R, typename SS, typename SP, int NM>
-PresArgs<R, SS, SP> pres_args(const fw_medium *m, const StepImages *im)
+PresArgs<R, SS, SP> pres_args(const fw_medium *m, const StepImages *im, const StepIo &io)
 {
     const StateAt at{static_cast<const char *>(m->slab), im};
     PresArgs<R, SS, SP> pa{};
@@ -220,6 +228,21 @@ PresArgs<R, SS, SP> pres_args(const fw_medium *m, const StepImages *im)
     pa.lut = static_cast<const R *>(m->lut);
     pa.mon = m->mon;
     pa.rho = static_cast<const SS *>(m->rho);
+    if (m->n_ent > 0) {
+        IoArgs<R, SS> &a = pa.io;
+        a.off = m->io_off;
+        a.ent = static_cast<const IoEntry *>(m->ent_buf);
+        a.gain = static_cast<const R *>(m->src_gain);
+        a.waves = static_cast<const R *>(m->waves);
+        a.wave_of = m->wave_of;
+        a.wave_len = m->n_src > 0 ? m->wave_len : 0;
+        a.traces = io.record && m->n_rcv > 0 ? static_cast<SS *>(m->traces) : nullptr;
+        a.n_rec = m->n_rec;
+        a.decim = m->decim;
+        a.d_it = io.d_it;
+        a.j = io.j;
+        a.vol = (long long)m->vol;
+    }
     return pa;
 }
 
@@ -240,7 +263,7 @@ PresArgs<R, SS, SP> pres_args(const fw_medium *m, const StepImages *im)
 constexpr int kTileMin = 2048, kTileLong = 16384;
 
 template <typename SP, int NM, bool TS>
-cudaError_t launch_tiles(const fw_medium *m, cudaStream_t s, int which, int gx, int n_tiles)
+cudaError_t launch_tiles(const fw_medium *m, cudaStream_t s, int which, int gx, int n_tiles, const StepIo &io)
 {
     constexpr int NS = 2;   // stages: the tile computed and the one on its way
     using LV = VelTile<SP, NM, TS>;
@@ -261,18 +284,18 @@ cudaError_t launch_tiles(const fw_medium *m, cudaStream_t s, int which, int gx, 
     if (which & 1)
         e = launch_kernel(kv, dim3(ctas), block, bv, s, pdl, vel_args<float, float, SP, NM>(m, nullptr), m->vel_maps, gx, run, rows);
     if (e == cudaSuccess && (which & 2))
-        e = launch_kernel(kp, dim3(ctas), block, bp, s, pdl, pres_args<float, float, SP, NM>(m, nullptr), m->pres_maps, gx, run, rows);
+        e = launch_kernel(kp, dim3(ctas), block, bp, s, pdl, pres_args<float, float, SP, NM>(m, nullptr, io), m->pres_maps, gx, run, rows);
     return e;
 }
 
 template <typename R, typename SS, typename SP, int NM, bool TS>
-cudaError_t launch_2d(const fw_medium *m, cudaStream_t s, int which, const StepImages *im)
+cudaError_t launch_2d(const fw_medium *m, cudaStream_t s, int which, const StepImages *im, const StepIo &io)
 {
     const int gx = (m->NX + 127) / 128;
     if constexpr (sizeof(R) == 4) {
         const long long n_tiles = (long long)gx * ((m->NZ + kTileH - 1) / kTileH);
-        if (which & 4) return launch_tiles<SP, NM, TS>(m, s, which, gx, 0);
-        if (m->tma && !im && n_tiles >= kTileMin && n_tiles < INT_MAX) return launch_tiles<SP, NM, TS>(m, s, which, gx, (int)n_tiles);
+        if (which & 4) return launch_tiles<SP, NM, TS>(m, s, which, gx, 0, io);
+        if (m->tma && !im && n_tiles >= kTileMin && n_tiles < INT_MAX) return launch_tiles<SP, NM, TS>(m, s, which, gx, (int)n_tiles, io);
     }
     if (which & 4) return cudaSuccess;
     const dim3 grid((unsigned)gx * (unsigned)((m->NZ + kPlaneBY - 1) / kPlaneBY)), block(32, kPlaneBY);
@@ -284,12 +307,12 @@ cudaError_t launch_2d(const fw_medium *m, cudaStream_t s, int which, const StepI
     if (e == cudaSuccess && (which & 2))
         e = launch_kernel(m->nonlinear ? k_pressure_plane<R, SS, SP, NM, kPlaneBY, true, TS>
                                        : k_pressure_plane<R, SS, SP, NM, kPlaneBY, false, TS>,
-                          grid, block, 0, s, pdl, pres_args<R, SS, SP, NM>(m, im), gx);
+                          grid, block, 0, s, pdl, pres_args<R, SS, SP, NM>(m, im, io), gx);
     return e;
 }
 
 template <typename R, typename SS, typename SP, int NM, bool TS, bool TMA>
-cudaError_t launch_3d_as(const fw_medium *m, cudaStream_t s, int which, const StepImages *im)
+cudaError_t launch_3d_as(const fw_medium *m, cudaStream_t s, int which, const StepImages *im, const StepIo &io)
 {
     constexpr int BX = Tile3<R>::BX, BYV = Tile3<R>::BYV, BYP = Tile3<R>::BYP;
     using LV = VelSmem<R, SS, SP, NM, BX, BYV, TS, TMA>;
@@ -325,7 +348,7 @@ cudaError_t launch_3d_as(const fw_medium *m, cudaStream_t s, int which, const St
                           vel_args<R, SS, SP, NM>(m, im), vm);
     if (e == cudaSuccess && (which & 2))
         e = launch_kernel(m->nonlinear ? kpn : kp, dim3(gx, (m->NY + BYP - 1) / BYP, segs(1)), dim3(BX, BYP), LP::bytes, s,
-                          pdl, pres_args<R, SS, SP, NM>(m, im), pm);
+                          pdl, pres_args<R, SS, SP, NM>(m, im, io), pm);
     return e;
 }
 
@@ -333,71 +356,60 @@ cudaError_t launch_3d_as(const fw_medium *m, cudaStream_t s, int which, const St
 // tensor maps for them (which address the medium's own arrays, so not for
 // image steps), by cp.async otherwise.
 template <typename R, typename SS, typename SP, int NM, bool TS>
-cudaError_t launch_3d(const fw_medium *m, cudaStream_t s, int which, const StepImages *im)
+cudaError_t launch_3d(const fw_medium *m, cudaStream_t s, int which, const StepImages *im, const StepIo &io)
 {
     if constexpr (sizeof(R) == 4) {
         if (which & 4) {   // both forms: image steps take the second one
-            const cudaError_t e = launch_3d_as<R, SS, SP, NM, TS, false>(m, s, which, im);
-            return e == cudaSuccess && m->tma ? launch_3d_as<R, SS, SP, NM, TS, true>(m, s, which, im) : e;
+            const cudaError_t e = launch_3d_as<R, SS, SP, NM, TS, false>(m, s, which, im, io);
+            return e == cudaSuccess && m->tma ? launch_3d_as<R, SS, SP, NM, TS, true>(m, s, which, im, io) : e;
         }
-        if (m->tma && !im) return launch_3d_as<R, SS, SP, NM, TS, true>(m, s, which, im);
+        if (m->tma && !im) return launch_3d_as<R, SS, SP, NM, TS, true>(m, s, which, im, io);
     }
-    return launch_3d_as<R, SS, SP, NM, TS, false>(m, s, which, im);
+    return launch_3d_as<R, SS, SP, NM, TS, false>(m, s, which, im, io);
 }
 
 template <typename R, typename SS, typename SP, bool TS>
-cudaError_t launch_ts(const fw_medium *m, cudaStream_t s, int which, const StepImages *im)
+cudaError_t launch_ts(const fw_medium *m, cudaStream_t s, int which, const StepImages *im, const StepIo &io)
 {
     const bool d3 = m->ndim == 3;
     switch (m->nmech) {
-    case 1: return d3 ? launch_3d<R, SS, SP, 1, TS>(m, s, which, im) : launch_2d<R, SS, SP, 1, TS>(m, s, which, im);
-    case 2: return d3 ? launch_3d<R, SS, SP, 2, TS>(m, s, which, im) : launch_2d<R, SS, SP, 2, TS>(m, s, which, im);
-    case 3: return d3 ? launch_3d<R, SS, SP, 3, TS>(m, s, which, im) : launch_2d<R, SS, SP, 3, TS>(m, s, which, im);
-    case 4: return d3 ? launch_3d<R, SS, SP, 4, TS>(m, s, which, im) : launch_2d<R, SS, SP, 4, TS>(m, s, which, im);
+    case 1: return d3 ? launch_3d<R, SS, SP, 1, TS>(m, s, which, im, io) : launch_2d<R, SS, SP, 1, TS>(m, s, which, im, io);
+    case 2: return d3 ? launch_3d<R, SS, SP, 2, TS>(m, s, which, im, io) : launch_2d<R, SS, SP, 2, TS>(m, s, which, im, io);
+    case 3: return d3 ? launch_3d<R, SS, SP, 3, TS>(m, s, which, im, io) : launch_2d<R, SS, SP, 3, TS>(m, s, which, im, io);
+    case 4: return d3 ? launch_3d<R, SS, SP, 4, TS>(m, s, which, im, io) : launch_2d<R, SS, SP, 4, TS>(m, s, which, im, io);
     default: return cudaErrorInvalidValue;
     }
 }
 
-// leapfrog instances, or those of the time-space stencil (time_order 4)
+// leapfrog instances, or those of the time-space stencil (time_order 4); the
+// pressure sweep of step *d_it + j of the medium's counter injects and records
 template <typename R, typename SS, typename SP>
-cudaError_t launch_sweeps(const fw_medium *m, cudaStream_t s, int which, const StepImages *im = nullptr)
+cudaError_t launch_sweeps(const fw_medium *m, cudaStream_t s, int which, const StepImages *im, const StepIo &io)
 {
-    return m->time_order == 4 ? launch_ts<R, SS, SP, true>(m, s, which, im)
-                              : launch_ts<R, SS, SP, false>(m, s, which, im);
+    return m->time_order == 4 ? launch_ts<R, SS, SP, true>(m, s, which, im, io)
+                              : launch_ts<R, SS, SP, false>(m, s, which, im, io);
+}
+
+template <typename R, typename SS, typename SP>
+cudaError_t launch_step_sweeps(const fw_medium *m, cudaStream_t s, int which, int j)
+{
+    return launch_sweeps<R, SS, SP>(m, s, which, nullptr, StepIo{m->d_it, j, true});
 }
 
 // One leapfrog step from the state image at im.rd into the one at
 // im.rd + im.wofs (both laid out as the medium's state), sources included at
-// step it (absolute); receivers are not recorded and the images' step
-// counters are not used.  For the adjoint's recomputation: no copy of the
-// state per step, the medium's own state untouched.
+// step it (absolute), receivers with record; the images' step counters are not
+// used (zero: a counter that holds 0).  For the adjoint: no copy of the state
+// per step, the medium's own state untouched.
 template <typename R, typename SS>
-cudaError_t launch_image_step(const fw_medium *m, const StepImages &im, const int *zero, int it, bool pdl, cudaStream_t s)
+cudaError_t launch_image_step(const fw_medium *m, const StepImages &im, const int *zero, int it, bool record, bool pdl,
+                              cudaStream_t s)
 {
-    cudaError_t e = cudaSuccess;
-    if (pdl) {
-        e = launch_sweeps<R, SS, SS>(m, s, 3, &im);
-    } else {                       // first kernel after an event of another stream
-        e = launch_sweeps<R, SS, SS>(m, s, 1 | 8, &im);
-        if (e == cudaSuccess) e = launch_sweeps<R, SS, SS>(m, s, 2, &im);
-    }
-    if (e != cudaSuccess || m->n_src <= 0) return e;
-    SS *p = reinterpret_cast<SS *>(const_cast<char *>(im.rd) + im.wofs +
-                                   (static_cast<const char *>(m->p) - static_cast<const char *>(m->slab)));
-    return launch_kernel(k_sources<SS, R>, dim3((m->n_src + 255) / 256), dim3(256), 0, s, true, p, m->src_idx,
-                         static_cast<const R *>(m->src_gain), m->wave_of, static_cast<const R *>(m->waves), m->wave_len,
-                         m->n_src, zero, it, (long long)m->vol, m->mon);
-}
-
-template <typename R, typename SS>
-cudaError_t launch_io(const fw_medium *m, int j, bool pdl, cudaStream_t s)
-{
-    const int n = m->n_src + m->n_rcv;
-    if (n <= 0) return cudaSuccess;
-    return launch_kernel(k_io<SS, R>, dim3((n + 255) / 256), dim3(256), 0, s, pdl, static_cast<SS *>(m->p), m->src_idx,
-                         static_cast<const R *>(m->src_gain), m->wave_of, static_cast<const R *>(m->waves), m->wave_len,
-                         m->n_src, m->src_rcv, m->rcv_idx, m->rcv_src, static_cast<SS *>(m->traces), m->n_rcv, m->n_rec,
-                         m->decim, m->d_it, j, (long long)m->vol, m->mon);
+    const StepIo io{zero, it, record};
+    if (pdl) return launch_sweeps<R, SS, SS>(m, s, 3, &im, io);
+    // first kernel after an event of another stream
+    const cudaError_t e = launch_sweeps<R, SS, SS>(m, s, 1 | 8, &im, io);
+    return e == cudaSuccess ? launch_sweeps<R, SS, SS>(m, s, 2, &im, io) : e;
 }
 
 }  // namespace fwgb

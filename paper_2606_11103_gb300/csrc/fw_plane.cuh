@@ -244,6 +244,11 @@ k_pressure_plane(const __grid_constant__ PresArgs<R, SS, SP> A, int gx)
     const Geo<R> &G = A.g;
     const PlanePos P = plane_pos<BY>(G, gx);
     PMax<R> pmax;
+    int io0 = 0, io1 = 0;                          // this tile's sources and receivers
+    if (A.io.off) {
+        io0 = __ldg(A.io.off + blockIdx.x);
+        io1 = __ldg(A.io.off + blockIdx.x + 1);
+    }
     if (!P.on) {
         pdl_wait();
     } else {
@@ -306,6 +311,7 @@ k_pressure_plane(const __grid_constant__ PresArgs<R, SS, SP> A, int gx)
         }
         Io<SS>::st(wr_at(A.p + row, A.wofs), pv);
     }
+    if (io0 < io1) tile_io(A.io, wr_at(A.p, A.wofs), io0, io1, threadIdx.y * 32 + threadIdx.x, 32 * BY, A.mon);
     record_max(A.mon, pmax);
 }
 
@@ -346,11 +352,12 @@ template <typename SP, int NM, bool NL, bool TS> struct PresTile {
 
 // The walk of a CTA over its run of tiles (gx strips, n_rows tiles per strip):
 // load(warp, position, stage, barrier) arms the barrier with the bytes of the
-// warp's share of a tile's copies and issues them NS - 1 tiles ahead, body(position, stage, wait) computes it in all.  Waits are
+// warp's share of a tile's copies and issues them NS - 1 tiles ahead,
+// body(position, stage, wait) computes it in all, after() follows it.  Waits are
 // bounded; after a timeout the sweep is flagged on the monitor.
-template <int NS, size_t STAGE, typename Load, typename Body>
+template <int NS, size_t STAGE, typename Load, typename Body, typename After>
 __device__ __forceinline__ void walk_tiles(unsigned char *smem, int gx, int run, int n_rows, Monitor *mon, const Load &load,
-                                           const Body &body)
+                                           const Body &body, const After &after)
 {
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + NS * STAGE);
     const bool lead = threadIdx.x == 0 && threadIdx.y < 3;   // three warps issue a share of the copies each
@@ -376,6 +383,7 @@ __device__ __forceinline__ void walk_tiles(unsigned char *smem, int gx, int run,
         body(xb, (r0 + i) * kTileH, smem + (i % NS) * STAGE, [&] {
             if (!timed_out && !mbar_wait_bounded(bars + i % NS, (unsigned)(i / NS) & 1u)) timed_out = true;
         });
+        after();
     }
     if (timed_out) {
         // record it and give the copies in flight one more bounded chance to
@@ -473,7 +481,7 @@ k_velocity_tiles(const __grid_constant__ VelArgs<float, float, SP> A, const __gr
 #pragma unroll
             for (int m = 0; m < NM; ++m) Io<SP>::st(A.psi[m][ax] + P.row, ps[m]);
         }
-    });
+    }, [] {});
 }
 
 template <typename SP, int NM, bool NL, bool TS, int NS>
@@ -506,6 +514,7 @@ k_pressure_tiles(const __grid_constant__ PresArgs<float, float, SP> A, const __g
             for (int m = 0; m < NM; ++m) tma_load_3d(st + L::o_psi + m * kTileN * sizeof(SP), &M.psi[m], xb, 0, zb, bar);
         }
     };
+    int io0 = 0, io1 = 0;                          // the tile's sources and receivers
     walk_tiles<NS, L::stage>(smem, gx, run, n_rows, A.mon, load, [&](int xb, int zb, unsigned char *st, auto wait) {
         PlanePos P;
         P.x0 = xb + 4 * tx;
@@ -513,6 +522,11 @@ k_pressure_tiles(const __grid_constant__ PresArgs<float, float, SP> A, const __g
         P.on = P.x0 < G.nx && P.z < G.nz;
         P.row = (long long)P.z * G.px + P.x0;
         const int x0 = P.x0, z = P.z;
+        if (A.io.off) {
+            const int *o = A.io.off + (long long)(zb / kTileH) * gx + xb / kTileW;
+            io0 = __ldg(o);
+            io1 = __ldg(o + 1);
+        }
         const bool in[3] = {P.on && G.wabs > 0 && (x0 < G.wabs || x0 + 3 >= G.nx - G.wabs), false,
                             P.on && G.wabs > 0 && (z < G.wabs || z >= G.nz - G.wabs)};
         float pp[3][4];
@@ -570,6 +584,8 @@ k_pressure_tiles(const __grid_constant__ PresArgs<float, float, SP> A, const __g
             pmax.see(pv[e]);
         }
         Io<float>::st(A.p + P.row, pv);
+    }, [&] {
+        if (io0 < io1) tile_io(A.io, A.p, io0, io1, ty * 32 + tx, 128, A.mon);
     });
     record_max(A.mon, pmax);
 }

@@ -494,8 +494,8 @@ int fw_server_submit(fw_server *s, const fw_request *req, long long *id)
     // medium + upload staging (one dense map and the beta map at most) +
     // source and receiver buffers, each rounded to the arena's granule
     const size_t padded = (size_t)((r.grid.nx + 31) / 32 * 32) * r.grid.ny * r.grid.nz;
-    j->footprint = bytes + padded * 8 + (size_t)n_src * 16 + (size_t)r.n_wave * r.n_steps * 8 +
-                   (size_t)n_rcv * (8 + 4 * n_rec) + (16u << 20);
+    j->footprint = bytes + padded * 8 + (size_t)n_src * 36 + (size_t)r.n_wave * r.n_steps * 8 +
+                   (size_t)n_rcv * (28 + 4 * n_rec) + (16u << 20);
     std::lock_guard<std::mutex> lk(s->mu);
     j->id = s->next_id++;
     j->t_submit = s->now();
