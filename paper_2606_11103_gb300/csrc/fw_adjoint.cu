@@ -38,6 +38,7 @@
 #include <vector>
 
 namespace fwgb {
+cudaError_t launch_advance(int *d_it, int n, bool pdl, cudaStream_t s);
 void *device_alloc(size_t bytes);
 void device_free(void *p);
 size_t state_image_bytes(const fw_medium *m);
@@ -454,7 +455,8 @@ int nblocks(long long n) { return (int)std::min<long long>((n + 255) / 256, 152L
 
 struct Buf {
     void *p = nullptr;
-    explicit Buf(size_t b) : p(b ? device_alloc(b) : nullptr) {}
+    size_t bytes;
+    explicit Buf(size_t b) : p(b ? device_alloc(b) : nullptr), bytes(b) {}
     ~Buf() { device_free(p); }
     Buf(const Buf &) = delete;
     Buf &operator=(const Buf &) = delete;
@@ -565,14 +567,43 @@ int gradient_impl(fw_medium *m, int n_steps, int K, const void *G, const void *a
         ADJ_CK(cudaStreamSynchronize(s));
     }
 
-    // ---- forward run with checkpoints ----
+    // ---- forward run ----
+    // The adjoint begins with the last two segments, whose images have buffers of
+    // their own (segs): their states are kept as the forward run passes them, by
+    // image steps, and only the segments before them are recomputed.
+    // (128 steps, K = 32: 62 recomputed steps instead of 124.)
     const long long it0 = m->step;
-    for (int k = 0; k < n_ck; ++k) {
-        ADJ_CK(cudaMemcpyAsync(static_cast<char *>(ck.p) + (size_t)k * SB, slab, SB, cudaMemcpyDeviceToDevice, s));
-        int rc = fw_run(m, std::min(K, n_steps - k * K), s);
-        if (rc) return rc;
+    const int n_run = std::max(0, n_ck - 2);      // segments run in place, recomputed later
+    char *segs[2] = {static_cast<char *>(seg0.p), static_cast<char *>(seg1.p)};
+    auto ck_at = [&](int si) { return static_cast<char *>(ck.p) + (size_t)si * SB; };
+    // One step from image rd to image wr (memory variables in the state type:
+    // FP32 or FP64 storage, the only ones fw_gradient accepts)
+    auto image_step = [&](const char *rd, char *wr, int k, bool record, bool pdl, cudaStream_t st) -> cudaError_t {
+        const StepImages im{rd, (long long)(wr - rd)};
+        const int *z = static_cast<const int *>(zero.p);
+        return sizeof(R) == 8 ? image_step_f64(m, im, z, (int)(it0 + k), record, pdl, st)
+                              : image_step_f32(m, im, z, (int)(it0 + k), record, pdl, st);
+    };
+    // image steps do not write the padding of a row, and read it as zero
+    if (m->px != m->NX)
+        for (Buf *b : {&ck, &fin, &seg0, &seg1})
+            if (b->p) ADJ_CK(cudaMemsetAsync(b->p, 0, b->bytes, s));
+    for (int si = 0; si < n_ck; ++si) {
+        const int k0 = si * K, k1 = std::min(n_steps, k0 + K);
+        if (si <= n_run) ADJ_CK(cudaMemcpyAsync(ck_at(si), slab, SB, cudaMemcpyDeviceToDevice, s));
+        if (si < n_run) {
+            int rc = fw_run(m, k1 - k0, s);
+            if (rc) return rc;
+            continue;
+        }
+        const char *rd = ck_at(si);
+        for (int k = k0; k < k1; ++k) {
+            char *wr = k + 1 < k1 ? segs[si & 1] + (size_t)(k - k0) * SB
+                                  : (si + 1 < n_ck ? ck_at(si + 1) : static_cast<char *>(fin.p));
+            ADJ_CK(image_step(rd, wr, k, true, true, s));
+            rd = wr;
+        }
     }
-    ADJ_CK(cudaMemcpyAsync(fin.p, slab, SB, cudaMemcpyDeviceToDevice, s));
 
     // ---- kernel arguments (pointers into images are set per step) ----
     AdjArgs<R> A{};
@@ -650,43 +681,31 @@ int gradient_impl(fw_medium *m, int n_steps, int K, const void *G, const void *a
         ss.ev.push_back(*e);
     }
     bool rev_recorded[2] = {false, false};
-    char *segs[2] = {static_cast<char *>(seg0.p), static_cast<char *>(seg1.p)};
     // images after steps k0 .. k1-2 of segment si into segs[si & 1]: each step
     // reads the image before it (the checkpoint first) and writes the next
-    // (the image step takes memory variables in the state type: FP32 or FP64
-    // storage, the only ones fw_gradient accepts)
     auto recompute = [&](int si) -> int {
         const int k0 = si * K, k1 = std::min(n_steps, k0 + K);
-        const char *rd = static_cast<const char *>(ck.p) + (size_t)si * SB;
+        const char *rd = ck_at(si);
         for (int k = k0; k < k1 - 1; ++k) {
             char *wr = segs[si & 1] + (size_t)(k - k0) * SB;
-            const StepImages im{rd, (long long)(wr - rd)};
-            const int itk = (int)(it0 + k);
-            if ((sizeof(R) == 8 ? image_step_f64(m, im, static_cast<const int *>(zero.p), itk, false, k > k0, ss.side)
-                                : image_step_f32(m, im, static_cast<const int *>(zero.p), itk, false, k > k0, ss.side)) != cudaSuccess)
-                return FW_ERR_CUDA;
+            if (image_step(rd, wr, k, false, k > k0, ss.side) != cudaSuccess) return FW_ERR_CUDA;
             rd = wr;
         }
         return FW_OK;
     };
     ADJ_CK(cudaEventRecord(ev_start, s));   // the forward run and the checkpoints
     ADJ_CK(cudaStreamWaitEvent(ss.side, ev_start, 0));
-    {
-        int rc = recompute(n_ck - 1);
-        if (rc) return rc;
-    }
-    ADJ_CK(cudaEventRecord(rec_done[(n_ck - 1) & 1], ss.side));
     for (int si = n_ck - 1; si >= 0; --si) {
         const int k0 = si * K, k1 = std::min(n_steps, k0 + K);
-        ADJ_CK(cudaStreamWaitEvent(s, rec_done[si & 1], 0));
-        if (si >= 1) {
+        if (si < n_run) ADJ_CK(cudaStreamWaitEvent(s, rec_done[si & 1], 0));
+        if (si >= 1 && si - 1 < n_run) {
             // segs[(si - 1) & 1] was last read by the adjoint of segment si + 1
             if (rev_recorded[(si + 1) & 1]) ADJ_CK(cudaStreamWaitEvent(ss.side, rev_done[(si + 1) & 1], 0));
             int rc = recompute(si - 1);
             if (rc) return rc;
             ADJ_CK(cudaEventRecord(rec_done[(si - 1) & 1], ss.side));
         }
-        const char *ck_si = static_cast<const char *>(ck.p) + (size_t)si * SB;
+        const char *ck_si = ck_at(si);
         // image j of the segment: the state after step k0 + j - 1
         auto image = [&](int j) -> const char * {
             if (j == 0) return ck_si;
@@ -716,8 +735,11 @@ int gradient_impl(fw_medium *m, int n_steps, int K, const void *G, const void *a
     }
     ADJ_CK(cudaEventRecord(side_done, ss.side));
     ADJ_CK(cudaStreamWaitEvent(s, side_done, 0));
-    // leave the medium at the end of the forward run
-    ADJ_CK(cudaMemcpyAsync(slab, fin.p, SB, cudaMemcpyDeviceToDevice, s));
+    // leave the medium at the end of the forward run: the fields of the last
+    // image, the step counter past the image steps (images hold no counters; the
+    // monitor has followed every step)
+    ADJ_CK(cudaMemcpyAsync(slab, fin.p, off(m->d_it), cudaMemcpyDeviceToDevice, s));
+    ADJ_CK(launch_advance(m->d_it, n_steps - n_run * K, false, s));
     m->step = it0 + n_steps;
 
     // ---- fold onto the user's grid and convert ----
