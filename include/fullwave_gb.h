@@ -297,7 +297,7 @@ int fw_read_receivers_range(fw_medium *m, int col0, int ncol, void *dst, void *s
  * unpadded C order, as float (as_f64 = 0) or double (as_f64 = 1); 16-bit
  * memory variables come back in the units of the FP32 ones.  Ordered on
  * stream; blocking.  Device memory: one staging buffer of the field's size
- * from the installed allocator.  Errors: FW_ERR_ARG (field, idx, pointer),
+ * from the installed allocator, none when dst is memory of this device.  Errors: FW_ERR_ARG (field, idx, pointer),
  * FW_ERR_NOMEM, FW_ERR_CUDA. */
 int fw_read_field(fw_medium *m, int which, int idx, void *dst, int as_f64, void *stream);
 
@@ -369,7 +369,10 @@ int fw_load_state(fw_medium *m, const void *src, void *stream);
  * (as_f64 = 0) or double (as_f64 = 1), C order, host or device; grad_c or
  * grad_alpha0 may be NULL.  Device memory: ceil(n_steps/K) + 2(K - 1) + 2
  * state images (about fw_state_bytes each), 2D + 1 fields, 4 FP64 maps and
- * the two output maps, from the installed allocator, released before return.  The
+ * the two output maps, from the installed allocator; they are kept for the
+ * medium's next gradient if they take at most 8 GiB and a quarter of the
+ * device's free memory, and given back by fw_destroy_medium, by
+ * fw_set_allocator and when an allocation of the library fails.  The
  * recomputation of one segment runs on a stream of its own beside the
  * adjoint of the next.  Blocking.
  * Errors: FW_ERR_ARG, FW_ERR_UNSUPPORTED (nonlinear media, 16-bit storage, the

@@ -35,12 +35,13 @@
 
 #include <algorithm>
 #include <cmath>
+#include <initializer_list>
 #include <vector>
 
 namespace fwgb {
 cudaError_t launch_advance(int *d_it, int n, bool pdl, cudaStream_t s);
-void *device_alloc(size_t bytes);
-void device_free(void *p);
+void *workspace_take(fw_medium *m, size_t bytes);
+void workspace_give(fw_medium *m, void *p, size_t bytes);
 size_t state_image_bytes(const fw_medium *m);
 cudaError_t image_step_f32(const fw_medium *m, const StepImages &im, const int *zero, int it, bool record, bool pdl,
                            cudaStream_t s);
@@ -453,13 +454,40 @@ cudaError_t launch_reverse(const AdjArgs<R> &A, int ndim, int nmech, int side, b
 
 int nblocks(long long n) { return (int)std::min<long long>((n + 255) / 256, 152LL * 16); }
 
+// All device buffers of one gradient in one block: sized first (p null), then
+// placed in the medium's workspace
 struct Buf {
     void *p = nullptr;
-    size_t bytes;
-    explicit Buf(size_t b) : p(b ? device_alloc(b) : nullptr), bytes(b) {}
-    ~Buf() { device_free(p); }
+    size_t bytes, at = 0;
+    explicit Buf(size_t b) : bytes(b) {}
     Buf(const Buf &) = delete;
     Buf &operator=(const Buf &) = delete;
+};
+
+struct Workspace {
+    fw_medium *m;
+    cudaStream_t s;
+    void *p = nullptr;
+    size_t bytes = 0;
+    Workspace(fw_medium *m_, cudaStream_t s_) : m(m_), s(s_) {}
+    Workspace(const Workspace &) = delete;
+    Workspace &operator=(const Workspace &) = delete;
+    ~Workspace()
+    {
+        if (p) cudaStreamSynchronize(s);   // nothing of this call may still run in it
+        workspace_give(m, p, bytes);
+    }
+    bool place(std::initializer_list<Buf *> bufs)
+    {
+        for (Buf *b : bufs) {
+            b->at = bytes;
+            bytes += (b->bytes + 255) / 256 * 256;
+        }
+        p = workspace_take(m, bytes);
+        for (Buf *b : bufs)
+            if (p && b->bytes) b->p = static_cast<char *>(p) + b->at;
+        return p != nullptr;
+    }
 };
 
 #define ADJ_CK(call)                                   \
@@ -522,7 +550,10 @@ int gradient_impl(fw_medium *m, int n_steps, int K, const void *G, const void *a
     const size_t nG = (size_t)m->n_rcv * m->n_rec;
     Buf dG(nG * sizeof(R)), dA0(alpha0 ? n_user * (as_f64 ? 8 : 4) : 0);
     Buf dlut((size_t)m->n_classes * kDStride * sizeof(R)), zero(256);   // zero: step counter of the image steps
-    if (!lam.p || !ck.p || !seg0.p || (n_ck > 1 && !seg1.p) || !fin.p || !scratch.p || !gacc.p || !uacc.p || (nG && !dG.p) || (alpha0 && !dA0.p) || !dlut.p || !zero.p)
+    const size_t eb = as_f64 ? 8 : 4;
+    Buf out(2 * n_user * eb);
+    Workspace ws(m, s);
+    if (!ws.place({&lam, &ck, &fin, &seg0, &seg1, &scratch, &gacc, &uacc, &dG, &dA0, &dlut, &zero, &out}))
         return FW_ERR_NOMEM;
     ADJ_CK(cudaMemsetAsync(zero.p, 0, 256, s));
     ADJ_CK(cudaMemsetAsync(lam.p, 0, SB, s));
@@ -747,8 +778,6 @@ int gradient_impl(fw_medium *m, int n_steps, int K, const void *G, const void *a
     k_grad_fold<R><<<nblocks((long long)n_user), 256, 0, s>>>(A.gk, A.gs, A.rho, static_cast<const R *>(m->cdev),
                                                             m->dt, m->NX, m->NY, m->NZ, m->px, m->wabs, uc, us);
     ADJ_CK(cudaGetLastError());
-    Buf out(2 * n_user * (as_f64 ? 8 : 4));
-    if (!out.p) return FW_ERR_NOMEM;
     const float *a0f = alpha0 && !as_f64 ? static_cast<const float *>(dA0.p) : nullptr;
     const double *a0d = alpha0 && as_f64 ? static_cast<const double *>(dA0.p) : nullptr;
     if (as_f64) {
@@ -761,7 +790,6 @@ int gradient_impl(fw_medium *m, int n_steps, int K, const void *G, const void *a
                                                                    grad_c ? o : nullptr, grad_a ? o + n_user : nullptr);
     }
     ADJ_CK(cudaGetLastError());
-    const size_t eb = as_f64 ? 8 : 4;
     if (grad_c) ADJ_CK(cudaMemcpyAsync(grad_c, out.p, n_user * eb, cudaMemcpyDefault, s));
     if (grad_a)
         ADJ_CK(cudaMemcpyAsync(grad_a, static_cast<char *>(out.p) + n_user * eb, n_user * eb, cudaMemcpyDefault, s));

@@ -40,6 +40,11 @@ using namespace fwgb;
 namespace {
 
 cudaError_t launch_sweep(const fw_medium *m, cudaStream_t s, int which, int j = 0);
+}  // namespace
+namespace fwgb {
+static bool release_idle(fw_medium *only);
+}
+namespace {
 
 // ---- allocator --------------------------------------------------------------
 std::mutex g_alloc_mu;
@@ -56,10 +61,8 @@ struct ThreadHook {
 };
 thread_local ThreadHook t_hook;
 
-void *dev_alloc(size_t bytes)
+void *dev_alloc_once(size_t bytes)
 {
-    if (bytes == 0) bytes = 256;
-    if (t_hook.alloc) return t_hook.alloc(bytes, t_hook.ctx);
     std::lock_guard<std::mutex> lk(g_alloc_mu);
     if (g_alloc) return g_alloc(bytes, g_alloc_ctx);
     void *p = nullptr;
@@ -67,6 +70,15 @@ void *dev_alloc(size_t bytes)
         cudaGetLastError();
         return nullptr;
     }
+    return p;
+}
+
+void *dev_alloc(size_t bytes)
+{
+    if (bytes == 0) bytes = 256;
+    if (t_hook.alloc) return t_hook.alloc(bytes, t_hook.ctx);
+    void *p = dev_alloc_once(bytes);
+    if (!p && fwgb::release_idle(nullptr)) p = dev_alloc_once(bytes);
     return p;
 }
 
@@ -81,6 +93,82 @@ void dev_free(void *p)
     if (g_free) g_free(p, g_alloc_ctx);
     else cudaFree(p);
 }
+
+}  // namespace
+
+namespace fwgb {
+// ---- workspaces kept with their media -------------------------------------------
+// The last gradient's device buffers stay with the medium for its next gradient
+// (allocating and freeing the 3.3 GB of a 1024^2 gradient of 128 steps took 4.4
+// of its 15.2 ms): at most 8 GiB and a quarter of what the device has free.
+// Idle ones are given back when an allocation of the library fails, when the
+// allocator is changed, and with the medium.
+std::mutex g_ws_mu;
+std::vector<fw_medium *> g_ws_media;      // media that hold a workspace
+
+// take the idle workspaces out of the media (of one medium, or all)
+static std::vector<void *> take_idle(fw_medium *only)
+{
+    std::vector<void *> out;
+    std::lock_guard<std::mutex> lk(g_ws_mu);
+    for (size_t i = 0; i < g_ws_media.size();) {
+        fw_medium *m = g_ws_media[i];
+        if (m->ws_busy || (only && m != only)) {
+            ++i;
+            continue;
+        }
+        out.push_back(m->ws);
+        m->ws = nullptr;
+        m->ws_bytes = 0;
+        g_ws_media.erase(g_ws_media.begin() + (long)i);
+    }
+    return out;
+}
+
+static bool release_idle(fw_medium *only)
+{
+    const std::vector<void *> v = take_idle(only);
+    for (void *p : v) dev_free(p);
+    return !v.empty();
+}
+
+void *workspace_take(fw_medium *m, size_t bytes)
+{
+    {
+        std::lock_guard<std::mutex> lk(g_ws_mu);
+        if (m->ws && m->ws_bytes >= bytes) {
+            m->ws_busy = true;
+            return m->ws;
+        }
+    }
+    release_idle(m);
+    return dev_alloc(bytes);
+}
+
+void workspace_give(fw_medium *m, void *p, size_t bytes)
+{
+    if (!p) return;
+    size_t avail = 0, total = 0;
+    std::unique_lock<std::mutex> lk(g_ws_mu);
+    if (m->ws == p) {                       // reused: stays
+        m->ws_busy = false;
+        return;
+    }
+    lk.unlock();
+    if (t_hook.alloc || bytes > (8ULL << 30) || cudaMemGetInfo(&avail, &total) != cudaSuccess || bytes > avail / 4) {
+        cudaGetLastError();
+        dev_free(p);
+        return;
+    }
+    lk.lock();
+    m->ws = p;
+    m->ws_bytes = bytes;
+    m->ws_busy = false;
+    g_ws_media.push_back(m);
+}
+}  // namespace fwgb
+
+namespace {
 
 // RAII device buffer for temporaries
 struct DevBuf {
@@ -101,6 +189,19 @@ bool is_device_ptr(const void *p)
         return false;
     }
     return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
+}
+
+// device memory of the current device (managed memory stays with the copy
+// engines), aligned for elements of eb bytes
+bool writable_here(const void *p, size_t eb)
+{
+    cudaPointerAttributes at{};
+    int dev = -1;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return at.type == cudaMemoryTypeDevice && at.device == dev && reinterpret_cast<uintptr_t>(p) % eb == 0;
 }
 
 // 8th-order staggered weights: sum |c_m| sets the leapfrog stability limit
@@ -275,17 +376,37 @@ __global__ void k_cmax(const T *c, const uint16_t *cls, const double *ceff_scale
     }
 }
 
-// dense <-> padded copies for field I/O (element type conversion included)
-template <typename S, typename D>
-__global__ void k_unpad(D *dst, const S *src, int nx, int ny, int nz, int px, double scale)
+// dense <-> padded copies for field I/O (element type conversion included).
+// Reading: one row per warp pair, four elements of a thread in flight; the
+// scale is a template choice because FP64 arithmetic is slow on this GPU (the
+// product and conversions in FP64 for every element took 738 us at 512^3, the
+// plain copy 200).
+template <typename S, typename D, bool SCALED>
+__global__ void k_unpad(D *dst, const S *src, int nx, long long rows, int px, double scale)
 {
-    const long long n = (long long)nx * ny * nz;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x) {
-        int x = int(i % nx);
-        long long r = i / nx;
-        dst[i] = D(double(src[r * px + x]) * scale);
+    for (long long r = blockIdx.x * (long long)blockDim.y + threadIdx.y; r < rows;
+         r += (long long)gridDim.x * blockDim.y) {
+        const S *a = src + r * px;
+        D *d = dst + r * nx;
+#pragma unroll 4
+        for (int x = threadIdx.x; x < nx; x += blockDim.x) d[x] = SCALED ? D(double(a[x]) * scale) : D(a[x]);
     }
+}
+
+template <typename S, typename D>
+cudaError_t unpad(const fw_medium *m, const void *src, D *dst, double scale, cudaStream_t s)
+{
+    const long long rows = (long long)m->NY * m->NZ;
+    const dim3 block(64, 4), grid((unsigned)std::min<long long>((rows + 3) / 4, 152LL * 64));
+    if (scale == 1.0) k_unpad<S, D, false><<<grid, block, 0, s>>>(dst, static_cast<const S *>(src), m->NX, rows, m->px, scale);
+    else k_unpad<S, D, true><<<grid, block, 0, s>>>(dst, static_cast<const S *>(src), m->NX, rows, m->px, scale);
+    return cudaGetLastError();
+}
+
+template <typename S, typename D>
+__global__ void k_convert(D *dst, const S *src, size_t n)
+{
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) dst[i] = D(src[i]);
 }
 
 template <typename S, typename D>
@@ -567,6 +688,7 @@ void release(fw_medium *m)
     if (!m) return;
     drop_graphs(m);
     if (m->cap_stream) cudaStreamDestroy(m->cap_stream);
+    release_idle(m);
     dev_free(m->src_buf);
     dev_free(m->rcv_buf);
     dev_free(m->ent_buf);
@@ -625,17 +747,10 @@ int field_ptr(fw_medium *m, int which, int idx, void **ptr, int *kind)
 template <typename D>
 cudaError_t unpad_any(const fw_medium *m, void *src, int kind, D *dst, double scale, cudaStream_t s)
 {
-    const size_t n = (size_t)m->NX * m->NY * m->NZ;
-    int nb = grid_blocks(n);
-    if (kind == 0 || m->storage == FW_STORE_F32 || m->storage == FW_STORE_F64) {
-        if (m->es == 8) k_unpad<double, D><<<nb, 256, 0, s>>>(dst, (const double *)src, m->NX, m->NY, m->NZ, m->px, scale);
-        else k_unpad<float, D><<<nb, 256, 0, s>>>(dst, (const float *)src, m->NX, m->NY, m->NZ, m->px, scale);
-    } else if (m->storage == FW_STORE_BF16) {
-        k_unpad<__nv_bfloat16, D><<<nb, 256, 0, s>>>(dst, (const __nv_bfloat16 *)src, m->NX, m->NY, m->NZ, m->px, scale);
-    } else {
-        k_unpad<__half, D><<<nb, 256, 0, s>>>(dst, (const __half *)src, m->NX, m->NY, m->NZ, m->px, scale);
-    }
-    return cudaGetLastError();
+    if (kind == 0 || m->storage == FW_STORE_F32 || m->storage == FW_STORE_F64)
+        return m->es == 8 ? unpad<double, D>(m, src, dst, scale, s) : unpad<float, D>(m, src, dst, scale, s);
+    return m->storage == FW_STORE_BF16 ? unpad<__nv_bfloat16, D>(m, src, dst, scale, s)
+                                       : unpad<__half, D>(m, src, dst, scale, s);
 }
 
 template <typename S>
@@ -904,16 +1019,14 @@ int set_psi_reference(fw_medium *m, const float *waveforms, size_t wl)
 }  // namespace
 
 namespace fwgb {
-// device memory through the installed allocator, and the size of the state
-// image (the checkpoint image without the step counter), for the adjoint
-void *device_alloc(size_t bytes) { return dev_alloc(bytes); }
+// allocator of the calling thread (the serving runtime's arena)
 void set_thread_allocator(void *(*alloc)(size_t, void *), void (*release)(void *, void *), void *ctx)
 {
     t_hook.alloc = alloc;
     t_hook.release = release;
     t_hook.ctx = ctx;
 }
-void device_free(void *p) { dev_free(p); }
+// size of the state image (the checkpoint image without the step counter), for the adjoint
 size_t state_image_bytes(const fw_medium *m)
 {
     Dims d{m->ndim, m->NX, m->NY, m->NZ, m->px, m->es, m->eps, m->wabs, m->nmech, m->plane, m->vol, m->nonlinear};
@@ -954,6 +1067,7 @@ const char *fw_strerror(int code)
 
 void fw_set_allocator(void *(*alloc)(size_t, void *), void (*release_fn)(void *, void *), void *ctx)
 {
+    release_idle(nullptr);
     std::lock_guard<std::mutex> lk(g_alloc_mu);
     if (alloc && release_fn) {
         g_alloc = alloc;
@@ -1350,11 +1464,14 @@ int fw_read_field(fw_medium *m, int which, int idx, void *dst, int as_f64, void 
     const size_t n = (size_t)m->NX * m->NY * m->NZ;
     const size_t eb = as_f64 ? 8 : 4;
     const double scale = kind == 1 ? 1.0 / psi_scale_of(m, which == FW_FIELD_PSI1 ? 1 : 2) : 1.0;
-    DevBuf tmp(n * eb);
-    if (!tmp.p) return FW_ERR_NOMEM;
-    if (as_f64) FW_CK(unpad_any<double>(m, src, kind, (double *)tmp.p, scale, s));
-    else FW_CK(unpad_any<float>(m, src, kind, (float *)tmp.p, scale, s));
-    FW_CK(cudaMemcpyAsync(dst, tmp.p, n * eb, cudaMemcpyDefault, s));
+    // memory of this device is written directly; anything else through a buffer
+    const bool direct = writable_here(dst, eb);
+    DevBuf tmp(direct ? 0 : n * eb);
+    if (!direct && !tmp.p) return FW_ERR_NOMEM;
+    void *to = direct ? dst : tmp.p;
+    if (as_f64) FW_CK(unpad_any<double>(m, src, kind, (double *)to, scale, s));
+    else FW_CK(unpad_any<float>(m, src, kind, (float *)to, scale, s));
+    if (!direct) FW_CK(cudaMemcpyAsync(dst, tmp.p, n * eb, cudaMemcpyDefault, s));
     FW_CK(cudaStreamSynchronize(s));
     return FW_OK;
 }
@@ -1391,8 +1508,8 @@ int fw_read_receivers(fw_medium *m, void *dst, int as_f64, void *stream)
     } else {
         DevBuf tmp(n * eb);
         if (!tmp.p) return FW_ERR_NOMEM;
-        if (as_f64) k_unpad<float, double><<<grid_blocks(n), 256, 0, s>>>((double *)tmp.p, (const float *)m->traces, (int)n, 1, 1, (int)n, 1.0);
-        else k_unpad<double, float><<<grid_blocks(n), 256, 0, s>>>((float *)tmp.p, (const double *)m->traces, (int)n, 1, 1, (int)n, 1.0);
+        if (as_f64) k_convert<<<grid_blocks(n), 256, 0, s>>>((double *)tmp.p, (const float *)m->traces, n);
+        else k_convert<<<grid_blocks(n), 256, 0, s>>>((float *)tmp.p, (const double *)m->traces, n);
         FW_CK(cudaGetLastError());
         FW_CK(cudaMemcpyAsync(dst, tmp.p, n * eb, cudaMemcpyDefault, s));
         FW_CK(cudaStreamSynchronize(s));

@@ -139,6 +139,10 @@ struct fw_medium {
     // both index lists to rebuild them
     int *src_rcv = nullptr, *rcv_src = nullptr;
     std::vector<long long> h_src_idx, h_rcv_idx;
+    // device buffers of the last gradient, kept for the next (workspace_take)
+    void *ws = nullptr;
+    size_t ws_bytes = 0;
+    bool ws_busy = false;
     // bookkeeping
     long long step = 0;
     int sticky = 0;

@@ -64,3 +64,36 @@ def test_gradient_with_dirty_device_memory(shape, checkpoint):
     for a, b in zip(out[0], out[1]):
         assert np.array_equal(a, b)
     assert np.isfinite(out[1][0]).all() and np.abs(out[1][0]).max() > 0
+
+
+def test_workspace_is_kept_and_given_back():
+    """Gradients of one medium reuse their device buffers (also after a larger
+    one) and give the same result; the memory comes back with the medium."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import paper_2606_11103_gb300 as fw
+    shape, n = (300, 310), 24
+    prm = to_c(oracle_params(0.5, 1.1, 2, maxiter=60), fw)
+    one = np.ones(shape, np.float32)
+    src = np.zeros(shape, np.uint8)
+    src[20] = 1
+    rcv = np.zeros(shape, np.uint8)
+    rcv[30, ::5] = 1
+    G = np.random.default_rng(0).standard_normal((int(rcv.sum()), n)).astype(np.float32)
+    wave = np.sin(np.arange(n) * 0.4).astype(np.float32)[None] * 1e-6
+    torch.cuda.synchronize()
+    free0 = torch.cuda.mem_get_info()[0]
+    m = fw.Medium.from_classes(shape, 4e-5, 1540 * one, 1000 * one, np.zeros(shape, np.uint16), [prm], cfl=0.3, pml=8)
+    m.set_sources(src, wave)
+    m.set_receivers(rcv, n)
+    start = m.save_state()
+    out = []
+    for checkpoint in (6, 24, 6, 3):
+        m.load_state(start)
+        out.append(m.gradient(n, G, checkpoint=checkpoint))
+    for gc, ga in out[1:]:
+        assert np.array_equal(gc, out[0][0]) and np.array_equal(ga, out[0][1])
+    m.close()
+    torch.cuda.synchronize()
+    assert abs(torch.cuda.mem_get_info()[0] - free0) < 256 << 20     # the library's own code and staging array stay
