@@ -167,6 +167,10 @@ template <typename R, int DIM> __device__ __forceinline__ bool adj_in_layer(cons
     return c < A.wabs || last >= P.n[ax] - A.wabs;
 }
 
+// Lines of the arrays a kernel reads late, on their way into L2 from its first
+// instructions on (no registers held): 128^3, N = 2, one gradient 10.2 -> 9.8 ms
+__device__ __forceinline__ void prefetch(const void *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
 __device__ __forceinline__ void add4(double *p, const double (&v)[4])
 {
     double2 *q = reinterpret_cast<double2 *>(p);
@@ -193,6 +197,15 @@ __global__ void __launch_bounds__(32 * kAdjRows, sizeof(R) == 4 ? 4 : 1) k_adj_p
     }
     pdl_wait();
     if (!P.on) return;
+#pragma unroll
+    for (int ax = 0; ax < 3; ++ax)
+        if (DIM == 3 || ax != 1) prefetch(A.fv1[ax] + P.i);
+#pragma unroll
+    for (int m = 0; m < NM; ++m) {
+        prefetch(A.L.lpsi2[m] + P.i);
+        prefetch(A.fpsi2[m] + P.i);
+    }
+    prefetch(A.gk + P.i);
     Io<R>::ld(A.L.lp + P.i, lp);
     adj_diff<R, 0, false>(A, P, A.Gd[0], d);
 #pragma unroll
@@ -345,6 +358,19 @@ __global__ void __launch_bounds__(32 * kAdjRows, sizeof(R) == 4 ? 4 : 1) k_adj_v
     }
     pdl_wait();
     if (!P.on) return;
+#pragma unroll
+    for (int ax = 0; ax < 3; ++ax) {
+        if (DIM == 2 && ax == 1) continue;
+        prefetch(A.L.lv[ax] + P.i);
+        prefetch(A.Q[ax] + P.i);
+#pragma unroll
+        for (int m = 0; m < NM; ++m) {
+            prefetch(A.L.lpsi1[m][ax] + P.i);
+            prefetch(A.fpsi1[m][ax] + P.i);
+        }
+    }
+    prefetch(A.fp + P.i);
+    prefetch(A.gs + P.i);
     Io<R>::ld(A.gsp + P.i, gs);
     if (adj_in_layer<R, DIM>(A, P, 0) || adj_in_layer<R, DIM>(A, P, 1) || adj_in_layer<R, DIM>(A, P, 2))
 #pragma unroll
