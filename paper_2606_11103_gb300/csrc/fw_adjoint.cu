@@ -27,7 +27,7 @@
 //       adjoint of g_d (-D-), then the pressure adjoint (gives that of q_d);
 //   k_adj_velocity: the velocity adjoint (a stencil of the adjoint of q_d;
 //       gives that of g_d);
-// and between them k_adj_io, the transpose of injection and recording.
+// the first also takes the transpose of injection and recording on its tile.
 // Gradients accumulate in FP64.
 // The linear system only (no nonlinear factor); FP32 and FP64 media.
 #include "fw_internal.h"
@@ -78,30 +78,47 @@ template <typename R> struct AdjArgs {
     R *Q[3], *Gd[3];   // adjoints of q_d (this step) and of g_d (the later step, then this one)
     R *gsp;            // this step's pressure-side term of the gradient with respect to the d factor
     double *gk, *gs;
+    // transpose of injection and recording by the pressure kernel's CTAs: their
+    // cells' entries (IoEntry), ordered by tile (off null: none)
+    const int *off;
+    const IoEntry *ent;
+    const R *waves, *G;        // source waveforms; dL/dtraces [receiver][n_col]
+    const int *wave_of;
+    int wave_len, n_col;
+    int it, col;               // the step; trace column of the step before it (-1: not recorded)
+    double inv_dxd;
 };
 
 // A thread's quad: coordinates, row lengths and strides per kernel axis
 struct AdjPos {
     int c[3], n[3];
     long long st[3], i;
+    unsigned tile;     // of the entries of sources and receivers
     bool on;
 };
 
-constexpr int kAdjRows = 4;   // rows of quads per CTA (y in 3D, depth in 2D)
+// CTA tiles of the reverse step, those of the pressure sweep's sources and
+// receivers (io_tiling): 128 x 4 points in 2D, 64 x 8 (FP64: 64 x 4) in 3D
+template <typename R, int DIM> struct AdjCta {
+    static constexpr int BX = DIM == 3 ? 16 : 32, BY = DIM == 3 && sizeof(R) == 4 ? 8 : 4;
+};
 
 template <typename R, int DIM> __device__ __forceinline__ AdjPos adj_pos(const AdjArgs<R> &A)
 {
-    const unsigned gx = (unsigned)(A.nx + 127) / 128;
+    constexpr int BX = AdjCta<R, DIM>::BX, BY = AdjCta<R, DIM>::BY;
+    const unsigned gx = (unsigned)(A.nx + 4 * BX - 1) / (4 * BX);
     unsigned r = blockIdx.x / gx;
     AdjPos P;
-    P.c[0] = 4 * (int)((blockIdx.x % gx) * 32 + threadIdx.x);
+    P.c[0] = 4 * (int)((blockIdx.x % gx) * BX + threadIdx.x);
     if (DIM == 3) {
-        const unsigned gy = (unsigned)(A.ny + kAdjRows - 1) / kAdjRows;
-        P.c[1] = (int)(r % gy) * kAdjRows + threadIdx.y;
+        const unsigned gy = (unsigned)(A.ny + BY - 1) / BY;
+        P.c[1] = (int)(r % gy) * BY + threadIdx.y;
         P.c[2] = (int)(r / gy);
+        P.tile = ((r % gy) * gx + blockIdx.x % gx) * (unsigned)A.nz + r / gy;
     } else {
         P.c[1] = 0;
-        P.c[2] = (int)r * kAdjRows + threadIdx.y;
+        P.c[2] = (int)r * BY + threadIdx.y;
+        P.tile = blockIdx.x;
     }
     P.n[0] = A.nx; P.n[1] = A.ny; P.n[2] = A.nz;
     P.st[0] = 1; P.st[1] = A.px; P.st[2] = A.plane;
@@ -186,17 +203,10 @@ __device__ __forceinline__ void add4(double *p, const double (&v)[4])
 // per point each way, mostly L2 hits from one kernel to the next).
 // Registers are held to four CTAs of 128 threads per SM in FP32.
 template <typename R, int DIM, int NM>
-__global__ void __launch_bounds__(32 * kAdjRows, sizeof(R) == 4 ? 4 : 1) k_adj_pressure(const __grid_constant__ AdjArgs<R> A)
+__device__ __forceinline__ void adj_pressure_quad(const AdjArgs<R> &A, const AdjPos &P, const uint16_t (&cls)[4],
+                                                  const R (&kd)[4])
 {
-    const AdjPos P = adj_pos<R, DIM>(A);
-    uint16_t cls[4];
-    R lp[4], kd[4], q[3][4], div[4], d[4];
-    if (P.on) {
-        quad_classes(__ldg(reinterpret_cast<const uint2 *>(A.cls + P.i)), cls);
-        Io<R>::ldg(A.kdt + P.i, kd);
-    }
-    pdl_wait();
-    if (!P.on) return;
+    R lp[4], q[3][4], div[4], d[4];
 #pragma unroll
     for (int ax = 0; ax < 3; ++ax)
         if (DIM == 3 || ax != 1) prefetch(A.fv1[ax] + P.i);
@@ -286,6 +296,39 @@ __global__ void __launch_bounds__(32 * kAdjRows, sizeof(R) == 4 ? 4 : 1) k_adj_p
     add4(A.gk + P.i, gk);
 }
 
+template <typename R, int DIM, int NM>
+__global__ void __launch_bounds__(AdjCta<R, DIM>::BX * AdjCta<R, DIM>::BY, sizeof(R) == 4 ? 4 : 1) k_adj_pressure(const __grid_constant__ AdjArgs<R> A)
+{
+    const AdjPos P = adj_pos<R, DIM>(A);
+    uint16_t cls[4];
+    R kd[4];
+    int first = 0, last = 0;
+    if (P.on) {
+        quad_classes(__ldg(reinterpret_cast<const uint2 *>(A.cls + P.i)), cls);
+        Io<R>::ldg(A.kdt + P.i, kd);
+    }
+    if (A.off) {
+        first = __ldg(A.off + P.tile);
+        last = __ldg(A.off + P.tile + 1);
+    }
+    pdl_wait();
+    if (P.on) adj_pressure_quad<R, DIM, NM>(A, P, cls, kd);
+    if (first >= last) return;
+    // Transpose of injection and recording on the tile's cells, once their
+    // pressure adjoint and source-gain gradient are stored: the gradient of the
+    // gain of step it, then the adjoint of the earlier step's receiver.  (As a
+    // kernel of its own 5 to 8 us per reverse step, 1 to 4 thousand sources.)
+    __syncthreads();
+    constexpr int BX = AdjCta<R, DIM>::BX, BY = AdjCta<R, DIM>::BY;
+    for (int j = first + threadIdx.y * BX + threadIdx.x; j < last; j += BX * BY) {
+        const IoEntry e = A.ent[j];
+        const R l = A.L.lp[e.cell];
+        if (e.src >= 0 && A.it < A.wave_len)
+            A.gk[e.cell] += double(A.waves[(size_t)A.wave_of[e.src] * A.wave_len + A.it]) * double(l) * A.inv_dxd;
+        if (e.rcv >= 0 && A.col >= 0) A.L.lp[e.cell] = l + A.G[(size_t)e.rcv * A.n_col + A.col];
+    }
+}
+
 // velocity adjoint along ax; adds its terms to gs
 template <typename R, int DIM, int NM, int ax>
 __device__ __forceinline__ void adj_velocity_axis(const AdjArgs<R> &A, const AdjPos &P, const uint16_t (&cls)[4],
@@ -347,7 +390,7 @@ __device__ __forceinline__ void adj_velocity_axis(const AdjArgs<R> &A, const Adj
 }
 
 template <typename R, int DIM, int NM>
-__global__ void __launch_bounds__(32 * kAdjRows, sizeof(R) == 4 ? 4 : 1) k_adj_velocity(const __grid_constant__ AdjArgs<R> A)
+__global__ void __launch_bounds__(AdjCta<R, DIM>::BX * AdjCta<R, DIM>::BY, sizeof(R) == 4 ? 4 : 1) k_adj_velocity(const __grid_constant__ AdjArgs<R> A)
 {
     const AdjPos P = adj_pos<R, DIM>(A);
     uint16_t cls[4];
@@ -383,31 +426,13 @@ __global__ void __launch_bounds__(32 * kAdjRows, sizeof(R) == 4 ? 4 : 1) k_adj_v
     add4(A.gs + P.i, g);
 }
 
-// Transpose of injection and recording (k_io), in one launch after the
-// pressure adjoint of step it: threads [0, n_src) take the source-gain
-// gradient of step it (it < wave_len; it < 0: none) from the pressure adjoint
-// at the source's cell, then add the adjoint of the earlier step's receiver on
-// that cell (col >= 0: its trace column); threads [n_src, n_src + n_rcv) add
-// those of the other receivers.
+// adjoints of the last step's receivers (trace column col), before the first
+// reverse step
 template <typename R>
-__global__ void k_adj_io(R *lp, const long long *src_idx, const R *waves, const int *wave_of, int wave_len, int it,
-                         int n_src, const int *src_rcv, const long long *rcv_idx, const int *rcv_src, const R *G,
-                         int n_rcv, int n_col, int col, double inv_dxd, double *gk)
+__global__ void k_adj_receivers(R *lp, const IoEntry *ent, int n, const R *G, int n_col, int col)
 {
-    pdl_launch();
-    pdl_wait();
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t < n_src) {
-        const long long k = src_idx[t];
-        const int r = col >= 0 ? src_rcv[t] : -1;
-        const R l = lp[k];
-        if (it >= 0 && it < wave_len) gk[k] += double(waves[(size_t)wave_of[t] * wave_len + it]) * double(l) * inv_dxd;
-        if (r >= 0) lp[k] = l + G[(size_t)r * n_col + col];
-    } else if (col >= 0 && t < n_src + n_rcv) {
-        const int r = t - n_src;
-        if (rcv_src[r] >= 0) return;     // added by the thread of the source on its cell
-        lp[rcv_idx[r]] += G[(size_t)r * n_col + col];
-    }
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j < n && ent[j].rcv >= 0) lp[ent[j].cell] += G[(size_t)ent[j].rcv * n_col + col];
 }
 
 // internal gradients -> the user's grid (transpose of the layer inheritance)
@@ -457,11 +482,11 @@ __global__ void k_grad_out(const double *uc, const double *us, const float *a0f,
 template <typename R, int DIM, int NM>
 cudaError_t launch_reverse_n(const AdjArgs<R> &A, int side, bool pdl, cudaStream_t s)
 {
-    const unsigned gx = (unsigned)(A.nx + 127) / 128;
-    const unsigned rows = DIM == 3 ? (unsigned)(A.ny + kAdjRows - 1) / kAdjRows * (unsigned)A.nz
-                                   : (unsigned)(A.nz + kAdjRows - 1) / kAdjRows;
+    constexpr int BX = AdjCta<R, DIM>::BX, BY = AdjCta<R, DIM>::BY;
+    const unsigned gx = (unsigned)(A.nx + 4 * BX - 1) / (4 * BX);
+    const unsigned rows = DIM == 3 ? (unsigned)(A.ny + BY - 1) / BY * (unsigned)A.nz : (unsigned)(A.nz + BY - 1) / BY;
     return launch_kernel(side == 2 ? k_adj_pressure<R, DIM, NM> : k_adj_velocity<R, DIM, NM>, dim3(gx * rows),
-                         dim3(32, kAdjRows), 0, s, pdl, A);
+                         dim3(BX, BY), 0, s, pdl, A);
 }
 
 // one half of a reverse step (side 2: pressure, 1: velocity); instances per
@@ -712,18 +737,21 @@ int gradient_impl(fw_medium *m, int n_steps, int K, const void *G, const void *a
     auto column = [m](long long it) {
         return m->n_rcv > 0 && it % m->decim == 0 && it / m->decim < m->n_rec ? (int)(it / m->decim) : -1;
     };
-    // source gradient of step it (-1: none) and receivers' adjoints of trace column col
-    cudaError_t e_io = cudaSuccess;
-    auto adjoint_io = [&](long long it, int col) {
-        const int n_io = m->n_src + (col >= 0 ? m->n_rcv : 0);
-        if (n_io <= 0 || (col < 0 && (it < 0 || it >= m->wave_len))) return;
-        e_io = launch_kernel(k_adj_io<R>, dim3((n_io + 255) / 256), dim3(256), 0, s, true, A.L.lp, m->src_idx,
-                             static_cast<const R *>(m->waves), m->wave_of, m->wave_len, (int)it, m->n_src, m->src_rcv,
-                             m->rcv_idx, m->rcv_src, static_cast<const R *>(dG.p), m->n_rcv, m->n_rec, col, inv_dxd,
-                             A.gk);
-    };
-    adjoint_io(-1, column(it0 + n_steps - 1));   // the last step's receivers
-    ADJ_CK(e_io);
+    if (m->n_ent > 0) {
+        A.off = m->io_off;
+        A.ent = static_cast<const IoEntry *>(m->ent_buf);
+        A.waves = static_cast<const R *>(m->waves);
+        A.wave_of = m->wave_of;
+        A.wave_len = m->n_src > 0 ? m->wave_len : 0;
+        A.G = static_cast<const R *>(dG.p);
+        A.n_col = m->n_rec;
+        A.inv_dxd = inv_dxd;
+        const int col = column(it0 + n_steps - 1);
+        if (col >= 0) {
+            k_adj_receivers<R><<<(m->n_ent + 255) / 256, 256, 0, s>>>(A.L.lp, A.ent, m->n_ent, A.G, A.n_col, col);
+            ADJ_CK(cudaGetLastError());
+        }
+    }
 
     // ---- reverse sweep, one checkpoint segment at a time ----
     // The recomputation of segment si - 1 (a side stream, into the other of two
@@ -781,9 +809,9 @@ int gradient_impl(fw_medium *m, int n_steps, int K, const void *G, const void *a
             }
             for (int q = 0; q < m->nmech; ++q) A.fpsi2[q] = reinterpret_cast<const R *>(F + off(m->psi2[q]));
             // a segment's first kernel follows an event of the side stream: no early start
+            A.it = (int)it;
+            A.col = k > 0 ? column(it - 1) : -1;
             ADJ_CK(launch_reverse<R>(A, m->ndim, m->nmech, 2, k < k1 - 1, s));
-            adjoint_io(it, k > 0 ? column(it - 1) : -1);
-            ADJ_CK(e_io);
             ADJ_CK(launch_reverse<R>(A, m->ndim, m->nmech, 1, true, s));
         }
         ADJ_CK(cudaEventRecord(rev_done[si & 1], s));
