@@ -1563,7 +1563,7 @@ int fw_status(fw_medium *m, float *max_abs_p)
     FW_CK(cudaMemcpy(&h, m->mon, sizeof(Monitor), cudaMemcpyDeviceToHost));
     if (max_abs_p) std::memcpy(max_abs_p, &h.max_bits, 4);
     if (h.nonfinite) m->sticky = FW_ERR_UNSTABLE;
-    if (h.bad_index) m->sticky = FW_ERR_STATE;
+    if (h.bad_index || h.timeout) m->sticky = FW_ERR_STATE;
     return m->sticky;
 }
 
