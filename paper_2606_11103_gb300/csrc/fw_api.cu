@@ -136,7 +136,7 @@ void *workspace_take(fw_medium *m, size_t bytes)
 {
     {
         std::lock_guard<std::mutex> lk(g_ws_mu);
-        if (m->ws && m->ws_bytes >= bytes) {
+        if (m->ws && !m->ws_busy && m->ws_bytes >= bytes) {
             m->ws_busy = true;
             return m->ws;
         }
@@ -161,6 +161,11 @@ void workspace_give(fw_medium *m, void *p, size_t bytes)
         return;
     }
     lk.lock();
+    if (m->ws) {                            // another gradient's was kept meanwhile
+        lk.unlock();
+        dev_free(p);
+        return;
+    }
     m->ws = p;
     m->ws_bytes = bytes;
     m->ws_busy = false;
