@@ -186,7 +186,7 @@ def measured_peaks():
 
 def kernel_source_sha():
     h = hashlib.sha256()
-    for f in ("fw_kernels.cuh", "fw_launch.cuh"):
+    for f in ("fw_kernels.cuh", "fw_plane.cuh", "fw_launch.cuh"):
         with open(os.path.join(ROOT, "paper_2606_11103_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
