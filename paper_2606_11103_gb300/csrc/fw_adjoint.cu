@@ -670,6 +670,15 @@ int gradient_impl(fw_medium *m, int n_steps, int K, const void *G, const void *a
     if (m->px != m->NX)
         for (Buf *b : {&ck, &fin, &seg0, &seg1})
             if (b->p) ADJ_CK(cudaMemsetAsync(b->p, 0, b->bytes, s));
+    // The last image becomes the medium's state.  Steps write the absorbing-layer
+    // memories inside the layer only and nothing between the arrays: there it
+    // starts with what the medium holds (a copy of 16 MiB at 1024^2, of the whole
+    // image where the arrays' size leaves gaps between them).
+    const size_t state_end = off(m->d_it);
+    const size_t unwritten = vol * sizeof(R) % 256 ? 0 : m->psi1p[0] ? off(m->psi1p[0]) : state_end;
+    if (unwritten < state_end)
+        ADJ_CK(cudaMemcpyAsync(static_cast<char *>(fin.p) + unwritten, slab + unwritten, state_end - unwritten,
+                               cudaMemcpyDeviceToDevice, s));
     for (int si = 0; si < n_ck; ++si) {
         const int k0 = si * K, k1 = std::min(n_steps, k0 + K);
         if (si <= n_run) ADJ_CK(cudaMemcpyAsync(ck_at(si), slab, SB, cudaMemcpyDeviceToDevice, s));
@@ -823,7 +832,7 @@ int gradient_impl(fw_medium *m, int n_steps, int K, const void *G, const void *a
     // leave the medium at the end of the forward run: the fields of the last
     // image, the step counter past the image steps (images hold no counters; the
     // monitor has followed every step)
-    ADJ_CK(cudaMemcpyAsync(slab, fin.p, off(m->d_it), cudaMemcpyDeviceToDevice, s));
+    ADJ_CK(cudaMemcpyAsync(slab, fin.p, state_end, cudaMemcpyDeviceToDevice, s));
     ADJ_CK(launch_advance(m->d_it, n_steps - n_run * K, false, s));
     m->step = it0 + n_steps;
 
