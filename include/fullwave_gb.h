@@ -297,8 +297,9 @@ int fw_read_receivers_range(fw_medium *m, int col0, int ncol, void *dst, void *s
  * unpadded C order, as float (as_f64 = 0) or double (as_f64 = 1); 16-bit
  * memory variables come back in the units of the FP32 ones.  Ordered on
  * stream; blocking.  Device memory: one staging buffer of the field's size
- * from the installed allocator, none when dst is memory of this device.  Errors: FW_ERR_ARG (field, idx, pointer),
- * FW_ERR_NOMEM, FW_ERR_CUDA. */
+ * from the installed allocator, none when dst is memory of this device.
+ * Errors: FW_ERR_ARG (field, idx, pointer), FW_ERR_NOMEM, FW_ERR_CUDA (also
+ * a device allocation too small for the field, which is not written). */
 int fw_read_field(fw_medium *m, int which, int idx, void *dst, int as_f64, void *stream);
 
 /* fw_read_field without any device allocation.  No counterpart in the

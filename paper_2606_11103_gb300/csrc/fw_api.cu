@@ -196,17 +196,38 @@ bool is_device_ptr(const void *p)
     return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
 }
 
-// device memory of the current device (managed memory stays with the copy
-// engines), aligned for elements of eb bytes
-bool writable_here(const void *p, size_t eb)
+// Entry point of a driver function, looked up through the runtime (no link
+// against the driver library).  Null where it is not available.
+void *driver_entry(const char *name)
 {
+    void *p = nullptr;
+    cudaDriverEntryPointQueryResult q{};
+    if (cudaGetDriverEntryPointByVersion(name, &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+        q == cudaDriverEntryPointSuccess)
+        return p;
+    cudaGetLastError();
+    return nullptr;
+}
+
+// device memory of the current device (managed memory stays with the copy
+// engines), aligned for elements of eb bytes, all of [p, p + bytes) in one
+// allocation: a kernel may write it.  Anything else is left to a copy, which
+// checks its destination.
+bool writable_here(const void *p, size_t bytes, size_t eb)
+{
+    using RangeFn = CUresult (*)(CUdeviceptr *, size_t *, CUdeviceptr);
+    static const RangeFn range = reinterpret_cast<RangeFn>(driver_entry("cuMemGetAddressRange"));
     cudaPointerAttributes at{};
     int dev = -1;
     if (cudaPointerGetAttributes(&at, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
-    return at.type == cudaMemoryTypeDevice && at.device == dev && reinterpret_cast<uintptr_t>(p) % eb == 0;
+    const CUdeviceptr d = reinterpret_cast<CUdeviceptr>(p);
+    if (at.type != cudaMemoryTypeDevice || at.device != dev || d % eb != 0) return false;
+    CUdeviceptr base = 0;
+    size_t size = 0;
+    return range && range(&base, &size, d) == CUDA_SUCCESS && d - base <= size && bytes <= size - (d - base);
 }
 
 // 8th-order staggered weights: sum |c_m| sets the leapfrog stability limit
@@ -216,22 +237,10 @@ double stencil_abs_sum()
 }
 
 // ---- tensor maps for TMA staging ----------------------------------------------
-// The driver's tensor-map encoder, looked up once through the runtime (no
-// link against the driver library).  Null where it is not available.
+// The driver's tensor-map encoder, looked up once
 EncodeTiledFn tensor_map_encoder()
 {
-    static std::once_flag once;
-    static EncodeTiledFn fn = nullptr;
-    std::call_once(once, [] {
-        void *p = nullptr;
-        cudaDriverEntryPointQueryResult q{};
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
-                cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<EncodeTiledFn>(p);
-        else
-            cudaGetLastError();
-    });
+    static const EncodeTiledFn fn = reinterpret_cast<EncodeTiledFn>(driver_entry("cuTensorMapEncodeTiled"));
     return fn;
 }
 
@@ -1470,7 +1479,7 @@ int fw_read_field(fw_medium *m, int which, int idx, void *dst, int as_f64, void 
     const size_t eb = as_f64 ? 8 : 4;
     const double scale = kind == 1 ? 1.0 / psi_scale_of(m, which == FW_FIELD_PSI1 ? 1 : 2) : 1.0;
     // memory of this device is written directly; anything else through a buffer
-    const bool direct = writable_here(dst, eb);
+    const bool direct = writable_here(dst, n * eb, eb);
     DevBuf tmp(direct ? 0 : n * eb);
     if (!direct && !tmp.p) return FW_ERR_NOMEM;
     void *to = direct ? dst : tmp.p;
