@@ -94,3 +94,25 @@ def test_state_after_a_gradient_is_that_of_a_run(fw, dirty_memory, shape, pml, t
     for label, a, b in states_after_run_and_gradient(fw, shape, pml, transition, storage, checkpoint):
         assert np.array_equal(a, b), label
     assert not dirty_memory
+
+
+def test_sides_of_the_attenuation_gradient_add_up_in_fp64(fw):
+    """Each cell's terms of a step, one of the pressure and one of the velocity
+    update, are FP32 sums that are added up in FP64: after one step their sum
+    has more than FP32's 24 bits except where the terms' last bits happen to
+    allow it (random bits: well below 9 cells of 10)."""
+    shape = (12, 14, 40)
+    rng = np.random.default_rng(7)
+    dx = 1500.0 / 36e6
+    one = np.ones(shape, np.float32)
+    m = fw.Medium.from_classes(shape, dx, 1500 * one, 1000 * one, np.zeros(shape, np.uint16),
+                               [to_c(oracle_params(0.5, 1.1, 2, maxiter=60), fw)], dt=0.3 * dx / 1530)
+    rcv = np.ones(shape, np.uint8)
+    m.set_receivers(rcv, 1)
+    for w, count in ((fw.FW_FIELD_P, 1), (fw.FW_FIELD_V, 3), (fw.FW_FIELD_PSI1, 6), (fw.FW_FIELD_PSI2, 2)):
+        for k in range(count):
+            m.write_field(w, k, rng.standard_normal(shape).astype(np.float32))
+    _, ga = m.gradient(1, rng.standard_normal((int(rcv.sum()), 1)), checkpoint=1, f64=True)
+    m.close()
+    assert np.isfinite(ga).all() and np.all(ga != 0)
+    assert np.mean(ga != ga.astype(np.float32).astype(np.float64)) > 0.1
