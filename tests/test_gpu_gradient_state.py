@@ -48,7 +48,7 @@ def dirty_memory(fw):
     fw.lib().fw_set_allocator(C.cast(None, _lib.ALLOCFN), C.cast(None, _lib.FREEFN), None)
 
 
-def states_after_run_and_gradient(fw, shape, pml, transition, storage, checkpoint):
+def states_after_run_and_gradient(fw, shape, pml, transition, storage, checkpoint, n_mech=2):
     rng = np.random.default_rng(11)
     dx = 1500.0 / 36e6
     c = (1500 + 30 * rng.uniform(-1, 1, shape)).astype(np.float32)
@@ -60,14 +60,14 @@ def states_after_run_and_gradient(fw, shape, pml, transition, storage, checkpoin
     n = 24
     wave = np.sin(np.arange(n) * 0.4).astype(np.float32)[None] * 1e-6
     G = rng.standard_normal((int(rcv.sum()), n)).astype(np.float32)
-    prm = [to_c(oracle_params(a, y, 2, maxiter=60), fw) for a, y in ((0.5, 1.1), (0.9, 1.5))]
+    prm = [to_c(oracle_params(a, y, n_mech, maxiter=60), fw) for a, y in ((0.5, 1.1), (0.9, 1.5))]
     m = fw.Medium.from_classes(shape, dx, c, rho, rng.integers(0, 2, shape).astype(np.uint16), prm,
                                dt=0.3 * dx / 1530, pml=pml, transition=transition, storage=storage)
     m.set_sources(src, wave)
     m.set_receivers(rcv, n)
     nd = len(shape)
     names = [(fw.FW_FIELD_P, 0)] + [(fw.FW_FIELD_V, k) for k in range(nd)]
-    names += [(fw.FW_FIELD_PSI1, k) for k in range(2 * nd)] + [(fw.FW_FIELD_PSI2, k) for k in range(2)]
+    names += [(fw.FW_FIELD_PSI1, k) for k in range(n_mech * nd)] + [(fw.FW_FIELD_PSI2, k) for k in range(n_mech)]
     layer = [(w, k) for w in (fw.FW_FIELD_PSI1P, fw.FW_FIELD_PSI2P) for k in range(nd)] if pml else []
     m.write_field(fw.FW_FIELD_P, 0, (1e3 * rng.standard_normal(shape)).astype(np.float32))
     for w, k in layer:
@@ -94,6 +94,17 @@ def test_state_after_a_gradient_is_that_of_a_run(fw, dirty_memory, shape, pml, t
     for label, a, b in states_after_run_and_gradient(fw, shape, pml, transition, storage, checkpoint):
         assert np.array_equal(a, b), label
     assert not dirty_memory
+
+
+@pytest.mark.parametrize("shape,pml,transition,checkpoint,n_mech", [
+    ((1024, 1056), 9, 0, 7, 3), ((1024, 1056), 9, 4, 24, 4), ((1029, 1021), 7, 5, 9, 2), ((2049, 515), 0, 0, 7, 1),
+    ((1030, 1024), 11, 0, 24, 4), ((40, 72, 130), 6, 3, 7, 1), ((40, 72, 130), 6, 0, 7, 2), ((40, 72, 130), 5, 0, 24, 3),
+    ((40, 72, 130), 7, 0, 9, 4)])
+def test_state_after_a_gradient_of_staged_sweeps(fw, shape, pml, transition, checkpoint, n_mech):
+    """Planes from 2048 tiles on and volumes: a run takes the sweeps staged by
+    TMA, the gradient's last two segments the image steps."""
+    for label, a, b in states_after_run_and_gradient(fw, shape, pml, transition, "f32", checkpoint, n_mech):
+        assert np.array_equal(a, b), label
 
 
 def test_sides_of_the_attenuation_gradient_add_up_in_fp64(fw):
