@@ -370,10 +370,12 @@ int fw_load_state(fw_medium *m, const void *src, void *stream);
  * (as_f64 = 0) or double (as_f64 = 1), C order, host or device; grad_c or
  * grad_alpha0 may be NULL.  Device memory: ceil(n_steps/K) + 2(K - 1) + 2
  * state images (about fw_state_bytes each), 2D + 1 fields, 4 FP64 maps and
- * the two output maps, from the installed allocator; they are kept for the
- * medium's next gradient if they take at most 8 GiB and a quarter of the
- * device's free memory, and given back by fw_destroy_medium, by
- * fw_set_allocator and when an allocation of the library fails.  The
+ * the two output maps, from the installed allocator.  Without an installed
+ * allocator they are kept for the medium's next gradient as long as those of
+ * all media together take at most 8 GiB and a quarter of the device's free
+ * memory, and given back by fw_release_workspace, fw_destroy_medium,
+ * fw_set_allocator and when an allocation of the library fails; an installed
+ * allocator has them back before return.  The
  * recomputation of one segment runs on a stream of its own beside the
  * adjoint of the next.  Blocking.
  * Errors: FW_ERR_ARG, FW_ERR_UNSUPPORTED (nonlinear media, 16-bit storage, the
@@ -382,6 +384,11 @@ int fw_load_state(fw_medium *m, const void *src, void *stream);
  * FW_ERR_NOMEM, FW_ERR_CUDA, or the medium's sticky error. */
 int fw_gradient(fw_medium *m, int n_steps, int checkpoint_every, const void *G, const void *alpha0,
                 void *grad_c, void *grad_alpha0, int as_f64, void *stream);
+
+/* Give back the device memory that media keep between gradients: m's, or
+ * every medium's for NULL (for a caller whose own allocation has failed).  A
+ * gradient in progress keeps its own.  Returns FW_OK. */
+int fw_release_workspace(fw_medium *m);
 
 /* Stability monitor (the divergence of long runs counted in Sec. 4.6 and
  * Sec. 5.5: non-finite pressure): synchronises the

@@ -265,6 +265,10 @@ class Medium:
                                 ptrs[0], ptrs[1], int(bool(f64)), _stream(stream)), "fw_gradient")
         return out
 
+    def release_workspace(self):
+        """Give back the device memory kept from the last gradient for the next."""
+        check(lib().fw_release_workspace(self.h), "fw_release_workspace")
+
     def state_bytes(self):
         n = C.c_size_t()
         check(lib().fw_state_bytes(self.h, C.byref(n)), "fw_state_bytes")

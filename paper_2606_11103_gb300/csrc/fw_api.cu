@@ -42,7 +42,7 @@ namespace {
 cudaError_t launch_sweep(const fw_medium *m, cudaStream_t s, int which, int j = 0);
 }  // namespace
 namespace fwgb {
-static bool release_idle(fw_medium *only);
+bool release_idle(fw_medium *only);
 }
 namespace {
 
@@ -99,12 +99,16 @@ void dev_free(void *p)
 namespace fwgb {
 // ---- workspaces kept with their media -------------------------------------------
 // The last gradient's device buffers stay with the medium for its next gradient
-// (allocating and freeing the 3.3 GB of a 1024^2 gradient of 128 steps took 4.4
-// of its 15.2 ms): at most 8 GiB and a quarter of what the device has free.
-// Idle ones are given back when an allocation of the library fails, when the
-// allocator is changed, and with the medium.
+// (allocating and freeing the 4.2 GiB of a 1024^2 gradient of 128 steps took 4.4
+// of its 15.2 ms): those of all media together at most 8 GiB and a quarter of
+// what the device has free.  (Larger ones belong to longer gradients: 8.3 ms
+// for 14.4 GiB, 3000 steps at 1024^2, of 260 ms.)  Never from an allocator that the caller installed,
+// whose pool is the place to keep memory.  Idle ones are given back when an
+// allocation of the library fails, when an allocator is installed, on
+// fw_release_workspace and with the medium.
 std::mutex g_ws_mu;
 std::vector<fw_medium *> g_ws_media;      // media that hold a workspace
+size_t g_ws_bytes = 0;                    // of all of them
 
 // take the idle workspaces out of the media (of one medium, or all)
 static std::vector<void *> take_idle(fw_medium *only)
@@ -118,6 +122,7 @@ static std::vector<void *> take_idle(fw_medium *only)
             continue;
         }
         out.push_back(m->ws);
+        g_ws_bytes -= m->ws_bytes;
         m->ws = nullptr;
         m->ws_bytes = 0;
         g_ws_media.erase(g_ws_media.begin() + (long)i);
@@ -125,10 +130,10 @@ static std::vector<void *> take_idle(fw_medium *only)
     return out;
 }
 
-static bool release_idle(fw_medium *only)
+bool release_idle(fw_medium *only)
 {
     const std::vector<void *> v = take_idle(only);
-    for (void *p : v) dev_free(p);
+    for (void *p : v) cudaFree(p);            // kept ones come from cudaMalloc
     return !v.empty();
 }
 
@@ -154,21 +159,22 @@ void workspace_give(fw_medium *m, void *p, size_t bytes)
         m->ws_busy = false;
         return;
     }
-    lk.unlock();
-    if (t_hook.alloc || bytes > (8ULL << 30) || cudaMemGetInfo(&avail, &total) != cudaSuccess || bytes > avail / 4) {
-        cudaGetLastError();
-        dev_free(p);
-        return;
+    bool keep = !t_hook.alloc && !m->ws;
+    {
+        std::lock_guard<std::mutex> la(g_alloc_mu);
+        keep = keep && !g_alloc;
     }
-    lk.lock();
-    if (m->ws) {                            // another gradient's was kept meanwhile
+    keep = keep && cudaMemGetInfo(&avail, &total) == cudaSuccess && g_ws_bytes + bytes <= std::min<size_t>(8ULL << 30, avail / 4);
+    if (!keep) {
         lk.unlock();
+        cudaGetLastError();
         dev_free(p);
         return;
     }
     m->ws = p;
     m->ws_bytes = bytes;
     m->ws_busy = false;
+    g_ws_bytes += bytes;
     g_ws_media.push_back(m);
 }
 }  // namespace fwgb
@@ -1092,6 +1098,12 @@ void fw_set_allocator(void *(*alloc)(size_t, void *), void (*release_fn)(void *,
         g_free = nullptr;
         g_alloc_ctx = nullptr;
     }
+}
+
+int fw_release_workspace(fw_medium *m)
+{
+    release_idle(m);
+    return FW_OK;
 }
 
 int fw_medium_bytes(const fw_grid *g, int n_mech, int storage, int nonlinear, size_t *bytes)

@@ -35,6 +35,7 @@
 
 namespace fwgb {
 void set_thread_allocator(void *(*alloc)(size_t, void *), void (*release)(void *, void *), void *ctx);
+bool release_idle(fw_medium *only);
 }  // namespace fwgb
 
 namespace {
@@ -46,10 +47,11 @@ public:
     int init(size_t bytes)
     {
         size_ = (bytes + 255) / 256 * 256;
-        if (cudaMalloc(&base_, size_) != cudaSuccess) {
+        for (int i = 0; i < 2; ++i) {
+            if (cudaMalloc(&base_, size_) == cudaSuccess) break;
             cudaGetLastError();
             base_ = nullptr;
-            return FW_ERR_NOMEM;
+            if (i > 0 || !fwgb::release_idle(nullptr)) return FW_ERR_NOMEM;
         }
         free_[0] = size_;
         return FW_OK;
