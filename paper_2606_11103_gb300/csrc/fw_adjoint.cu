@@ -97,10 +97,9 @@ struct AdjPos {
     bool on;
 };
 
-// CTA tiles of the reverse step, those of the pressure sweep's sources and
-// receivers (io_tiling): 128 x 4 points in 2D, 64 x 8 (FP64: 64 x 4) in 3D
+// CTAs of the reverse step: the tiles of the sweeps' sources and receivers
 template <typename R, int DIM> struct AdjCta {
-    static constexpr int BX = DIM == 3 ? 16 : 32, BY = DIM == 3 && sizeof(R) == 4 ? 8 : 4;
+    static constexpr int BX = (DIM == 3 ? kTile3W : kTileW) / 4, BY = DIM == 3 ? tile3_rows(sizeof(R)) : kTileH;
 };
 
 template <typename R, int DIM> __device__ __forceinline__ AdjPos adj_pos(const AdjArgs<R> &A)

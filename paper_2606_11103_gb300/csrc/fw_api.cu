@@ -497,12 +497,12 @@ struct Dims {
 int axis_len(const Dims &d, int ax) { return ax == 0 ? d.NX : (ax == 1 ? d.NY : d.NZ); }
 bool axis_on(const Dims &d, int ax) { return !(d.ndim == 2 && ax == 1); }
 
-// tiles of the pressure sweep (fw_launch.cuh: Tile3 and the 2D tiles)
+// tiles of the pressure sweep
 IoTiling io_tiling(int ndim, int nx, int ny, int nz, int es)
 {
     IoTiling t{};
-    t.w = ndim == 3 ? 64 : 128;
-    t.h = ndim == 3 && es == 4 ? 8 : 4;
+    t.w = ndim == 3 ? kTile3W : kTileW;
+    t.h = ndim == 3 ? tile3_rows(es) : kTileH;
     t.gx = (nx + t.w - 1) / t.w;
     t.gy = ((ndim == 3 ? ny : nz) + t.h - 1) / t.h;
     t.n = (long long)t.gx * t.gy * (ndim == 3 ? nz : 1);
@@ -998,7 +998,8 @@ int create_common(const fw_grid *g, const float *c, const float *rho, const floa
     if (cudaStreamCreateWithFlags(&m->cap_stream, cudaStreamNonBlocking) != cudaSuccess) { release(m); return FW_ERR_CUDA; }
     if (launch_sweep(m, s, 4) != cudaSuccess) { release(m); return FW_ERR_CUDA; }
     if (m->ndim == 3) {
-        const long long tiles = ((m->NX + 63LL) / 64) * (m->es == 8 ? (m->NY + 3LL) / 4 : (m->NY + 7LL) / 8);
+        const IoTiling t = io_tiling(3, m->NX, m->NY, m->NZ, m->es);
+        const long long tiles = (long long)t.gx * t.gy;
         for (int i = 0; i < 2; ++i) m->zseg[i] = choose_zseg(tiles, m->NZ, m->slots[i]);
     }
     if (cudaStreamSynchronize(s) != cudaSuccess) { release(m); return FW_ERR_CUDA; }

@@ -77,6 +77,14 @@ struct IoEntry {
     int src, rcv;
 };
 
+// CTA tiles: columns, and rows of depth (2D) or y (3D, by the bytes of a state
+// element).  All sweeps and the reverse kernels take these: a cell's source or
+// receiver is handled, without atomics, by the CTA that stores the cell, found by
+// the tile it lies in.  A row of a 2D tile is a warp, a quad of columns per lane.
+constexpr int kTileW = 128, kTileH = 4;
+constexpr int kTile3W = 64;
+constexpr int tile3_rows(size_t es) { return es == 8 ? 4 : 8; }
+
 // Tiles of the pressure sweep's CTAs by kernel axes, in 3D one per depth plane,
 // the planes of a tile following each other; the entries of a medium's cells
 // are ordered by tile

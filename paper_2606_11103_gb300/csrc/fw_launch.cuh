@@ -37,9 +37,8 @@ cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, dim3 block, size_t sm
 // 360, 256^3 508 / 504 / 514, 256^3 binary16 391 / 374, 256^3 time-space 647 /
 // 623, 512^3 3822 / 3826.
 template <typename R> struct Tile3 {
-    static constexpr int BX = 16, BYV = sizeof(R) == 8 ? 4 : 8, BYP = BYV;
+    static constexpr int BX = kTile3W / 4, BYV = tile3_rows(sizeof(R)), BYP = BYV;
 };
-constexpr int kPlaneBY = 4;   // rows per CTA of the unstaged 2D sweeps
 
 template <typename R> Geo<R> make_geo(const fw_medium *m)
 {
@@ -276,7 +275,7 @@ cudaError_t launch_tiles(const fw_medium *m, cudaStream_t s, int which, int gx, 
         const cudaError_t e = cudaFuncSetAttribute(kv, attr, (int)bv);
         return e == cudaSuccess ? cudaFuncSetAttribute(kp, attr, (int)bp) : e;
     }
-    const dim3 block(32, kTileH);
+    const dim3 block(kTileW / 4, kTileH);
     const int run = n_tiles >= kTileLong ? 4 : 2;
     const int rows = n_tiles / gx, ctas = gx * ((rows + run - 1) / run);
     const bool pdl = !(which & 8);
@@ -291,22 +290,22 @@ cudaError_t launch_tiles(const fw_medium *m, cudaStream_t s, int which, int gx, 
 template <typename R, typename SS, typename SP, int NM, bool TS>
 cudaError_t launch_2d(const fw_medium *m, cudaStream_t s, int which, const StepImages *im, const StepIo &io)
 {
-    const int gx = (m->NX + 127) / 128;
+    const int gx = (m->NX + kTileW - 1) / kTileW;
     if constexpr (sizeof(R) == 4) {
         const long long n_tiles = (long long)gx * ((m->NZ + kTileH - 1) / kTileH);
         if (which & 4) return launch_tiles<SP, NM, TS>(m, s, which, gx, 0, io);
         if (m->tma && !im && n_tiles >= kTileMin && n_tiles < INT_MAX) return launch_tiles<SP, NM, TS>(m, s, which, gx, (int)n_tiles, io);
     }
     if (which & 4) return cudaSuccess;
-    const dim3 grid((unsigned)gx * (unsigned)((m->NZ + kPlaneBY - 1) / kPlaneBY)), block(32, kPlaneBY);
+    const dim3 grid((unsigned)gx * (unsigned)((m->NZ + kTileH - 1) / kTileH)), block(kTileW / 4, kTileH);
     const bool pdl = !(which & 8);
     cudaError_t e = cudaSuccess;
     if (which & 1)
-        e = launch_kernel(k_velocity_plane<R, SS, SP, NM, kPlaneBY, TS>, grid, block, 0, s, pdl,
+        e = launch_kernel(k_velocity_plane<R, SS, SP, NM, kTileH, TS>, grid, block, 0, s, pdl,
                           vel_args<R, SS, SP, NM>(m, im), gx);
     if (e == cudaSuccess && (which & 2))
-        e = launch_kernel(m->nonlinear ? k_pressure_plane<R, SS, SP, NM, kPlaneBY, true, TS>
-                                       : k_pressure_plane<R, SS, SP, NM, kPlaneBY, false, TS>,
+        e = launch_kernel(m->nonlinear ? k_pressure_plane<R, SS, SP, NM, kTileH, true, TS>
+                                       : k_pressure_plane<R, SS, SP, NM, kTileH, false, TS>,
                           grid, block, 0, s, pdl, pres_args<R, SS, SP, NM>(m, im, io), gx);
     return e;
 }

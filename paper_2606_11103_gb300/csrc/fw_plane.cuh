@@ -27,7 +27,7 @@ struct PlanePos {
 template <int BY, typename R> __device__ __forceinline__ PlanePos plane_pos(const Geo<R> &G, int gx)
 {
     PlanePos P;
-    P.x0 = 4 * (int)((blockIdx.x % gx) * 32 + threadIdx.x);
+    P.x0 = 4 * (int)((blockIdx.x % gx) * (kTileW / 4) + threadIdx.x);
     P.z = (int)(blockIdx.x / gx) * BY + threadIdx.y;
     P.on = P.x0 < G.nx && P.z < G.nz;
     P.row = (long long)P.z * G.px + P.x0;
@@ -322,7 +322,8 @@ k_pressure_plane(const __grid_constant__ PresArgs<R, SS, SP> A, int gx)
 // tiles down a strip of 128 columns and keeps NS - 1 of them in flight ahead
 // of the one it computes, each with its halos in one box per stream; nothing
 // is carried from tile to tile but the coefficients of the last classes.
-constexpr int kTileW = 128, kTileH = 4, kTileN = kTileW * kTileH;
+constexpr int kTileN = kTileW * kTileH;
+static_assert(kTileW == 4 * 32, "a warp per row: walk_tiles, tile_io");
 
 constexpr size_t pad128(size_t b) { return (b + 127) / 128 * 128; }
 
