@@ -618,8 +618,6 @@ std::vector<double> build_lut(const fw_medium *m)
     for (size_t c = 0; c < cl.size(); ++c) {
         const fw_relax_params &p = cl[c];
         double *e = &t[c * kLutStride];
-        e[0] = p.kappa1;
-        e[1] = p.kappa2;
         for (int m = 0; m < p.n_mech; ++m) {
             double b1 = std::exp(-(p.d1[m] / p.kappa1 + p.alpha1[m]) * dt);
             double a1 = p.d1[m] / (p.kappa1 * (p.d1[m] + p.kappa1 * p.alpha1[m])) * (b1 - 1.0);
@@ -1194,16 +1192,14 @@ int fw_create_medium(const fw_grid *g, const float *c, const float *rho, const f
     return create_common(g, c, rho, beta, idx.data(), classes, storage, (cudaStream_t)stream, out);
 }
 
-// The lists behind injection and recording, from the sorted cells of the
-// sources and of the receivers: which receiver shares a source's cell and the
-// reverse (the adjoint's kernel lets one thread handle such a cell), and the
-// pressure sweep's entries, one per cell, ordered by tile.  A list no longer
-// than the last one needs no device memory, so after a set has been dropped
-// this cannot fail for want of it.
+// The list behind injection and recording (and their transpose), from the
+// sorted cells of the sources and of the receivers: one entry per cell, so that
+// one thread handles a cell with both, ordered by tile.  A list no longer than
+// the last one needs no device memory, so after a set has been dropped this
+// cannot fail for want of it.
 static int upload_io_map(fw_medium *m, cudaStream_t s)
 {
     const std::vector<long long> &a = m->h_src_idx, &b = m->h_rcv_idx;
-    std::vector<int> sr(a.size(), -1), rs(b.size(), -1);
     std::vector<IoEntry> e;
     e.reserve(a.size() + b.size());
     for (size_t i = 0, j = 0; i < a.size() || j < b.size();) {
@@ -1214,8 +1210,6 @@ static int upload_io_map(fw_medium *m, cudaStream_t s)
             e.push_back({b[j], -1, (int)j});
             ++j;
         } else {
-            sr[i] = (int)j;
-            rs[j] = (int)i;
             e.push_back({a[i], (int)i, (int)j});
             ++i;
             ++j;
@@ -1244,8 +1238,6 @@ static int upload_io_map(fw_medium *m, cudaStream_t s)
         }
     }
     m->n_ent = 0;                  // no entries should a copy fail
-    if (m->src_rcv && !sr.empty()) FW_CK(cudaMemcpyAsync(m->src_rcv, sr.data(), sr.size() * 4, cudaMemcpyHostToDevice, s));
-    if (m->rcv_src && !rs.empty()) FW_CK(cudaMemcpyAsync(m->rcv_src, rs.data(), rs.size() * 4, cudaMemcpyHostToDevice, s));
     if (!e.empty()) {
         FW_CK(cudaMemcpyAsync(m->io_off, off.data(), off.size() * 4, cudaMemcpyHostToDevice, s));
         FW_CK(cudaMemcpyAsync(m->ent_buf, sorted.data(), sorted.size() * sizeof(IoEntry), cudaMemcpyHostToDevice, s));
@@ -1276,7 +1268,6 @@ int fw_set_sources(fw_medium *m, const uint8_t *mask, const float *waveforms, in
     drop_graphs(m);
     dev_free(m->src_buf);
     m->src_buf = nullptr;
-    m->src_rcv = nullptr;
     m->n_src = 0;
     m->h_src_idx.clear();
     // receivers stop pointing at the old sources before anything can fail
@@ -1284,15 +1275,13 @@ int fw_set_sources(fw_medium *m, const uint8_t *mask, const float *waveforms, in
     if (ns == 0) return FW_OK;
     const size_t wl = (size_t)n_wave * n_steps;
     const size_t o_idx = 0, o_gain = align_up(ns * 8, 256), o_wof = o_gain + align_up((size_t)ns * m->es, 256),
-                 o_map = o_wof + align_up((size_t)ns * 4, 256), o_wave = o_map + align_up((size_t)ns * 4, 256),
-                 total = o_wave + align_up(wl * m->es, 256);
+                 o_wave = o_wof + align_up((size_t)ns * 4, 256), total = o_wave + align_up(wl * m->es, 256);
     m->src_buf = dev_alloc(total);
     if (!m->src_buf) return FW_ERR_NOMEM;
     char *b = static_cast<char *>(m->src_buf);
     m->src_idx = reinterpret_cast<long long *>(b + o_idx);
     m->src_gain = b + o_gain;
     m->wave_of = reinterpret_cast<int *>(b + o_wof);
-    m->src_rcv = reinterpret_cast<int *>(b + o_map);
     m->waves = b + o_wave;
     // every upload is ordered on the medium's stream and complete before
     // return: later work on any other (non-blocking) stream reads these
@@ -1334,7 +1323,6 @@ int fw_set_receivers(fw_medium *m, const uint8_t *mask, int decim, int n_steps)
     drop_graphs(m);
     dev_free(m->rcv_buf);
     m->rcv_buf = nullptr;
-    m->rcv_src = nullptr;
     m->n_rcv = 0;
     m->n_rec = 0;
     m->h_rcv_idx.clear();
@@ -1343,16 +1331,10 @@ int fw_set_receivers(fw_medium *m, const uint8_t *mask, int decim, int n_steps)
     const int nr = (int)idx.size();
     if (nr == 0) return FW_OK;
     const int nrec = (n_steps + decim - 1) / decim;
-    const size_t o_map = align_up((size_t)nr * 8, 256), o_tr = o_map + align_up((size_t)nr * 4, 256),
-                 total = o_tr + align_up((size_t)nr * std::max(nrec, 1) * m->es, 256);
-    m->rcv_buf = dev_alloc(total);
+    m->rcv_buf = dev_alloc((size_t)nr * std::max(nrec, 1) * m->es);
     if (!m->rcv_buf) return FW_ERR_NOMEM;
-    char *b = static_cast<char *>(m->rcv_buf);
-    m->rcv_idx = reinterpret_cast<long long *>(b);
-    m->rcv_src = reinterpret_cast<int *>(b + o_map);
-    m->traces = b + o_tr;
+    m->traces = m->rcv_buf;
     // ordered on the medium's stream and complete before return (see fw_set_sources)
-    FW_CK(cudaMemcpyAsync(m->rcv_idx, idx.data(), nr * 8, cudaMemcpyHostToDevice, s));
     FW_CK(cudaMemsetAsync(m->traces, 0, (size_t)nr * std::max(nrec, 1) * m->es, s));
     FW_CK(cudaStreamSynchronize(s));
     m->n_rcv = nr;

@@ -29,12 +29,12 @@ int nelder_mead(int n, double *x, const double *lo, const double *hi,
                 double xatol, double fatol, double *fmin, int *n_iter, int *n_eval);
 
 // ---- device layout ---------------------------------------------------------
-constexpr int kLutStride = 24;   // values per class in the coefficient table
-// table block offsets (in values): 0 kappa1, 1 kappa2, 4.. a1[4], 8.. b1[4],
-// 12.. a2[4], 16.. b2[4], 20 1/kappa1, 21 what its rounding left off, 22, 23
-// the same of kappa2 (the remainders: FP32 media; both with the known rounding
-// of the global factors taken back, see build_lut)
-constexpr int kLutA1 = 4, kLutB1 = 8, kLutA2 = 12, kLutB2 = 16, kLutIk1 = 20, kLutIk2 = 22;
+constexpr int kLutStride = 20;   // values per class in the coefficient table
+// table block offsets (in values): 0.. a1[4], 4.. b1[4], 8.. a2[4], 12.. b2[4],
+// 16 1/kappa1, 17 what its rounding left off, 18, 19 the same of kappa2 (the
+// remainders: FP32 media; both with the known rounding of the global factors
+// taken back, see build_lut)
+constexpr int kLutA1 = 0, kLutB1 = 4, kLutA2 = 8, kLutB2 = 12, kLutIk1 = 16, kLutIk2 = 18;
 
 struct Monitor {
     unsigned int max_bits;   // bits of max |p| (non-negative float)
@@ -131,7 +131,7 @@ struct fw_medium {
     std::vector<fw_relax_params> classes;
     // sources / receivers
     void *src_buf = nullptr, *rcv_buf = nullptr;
-    long long *src_idx = nullptr, *rcv_idx = nullptr;
+    long long *src_idx = nullptr;
     void *src_gain = nullptr, *waves = nullptr, *traces = nullptr;
     int *wave_of = nullptr;
     int n_src = 0, n_wave = 0, wave_len = 0;
@@ -142,11 +142,7 @@ struct fw_medium {
     size_t ent_cap = 0;
     int n_ent = 0;
     int *io_off = nullptr;
-    // cells that hold both a source and a receiver: per source the receiver
-    // there (or -1), per receiver the source there (or -1); host copies of
-    // both index lists to rebuild them
-    int *src_rcv = nullptr, *rcv_src = nullptr;
-    std::vector<long long> h_src_idx, h_rcv_idx;
+    std::vector<long long> h_src_idx, h_rcv_idx;   // the sources' and the receivers' cells, sorted
     // device buffers of the last gradient, kept for the next (workspace_take)
     void *ws = nullptr;
     size_t ws_bytes = 0;

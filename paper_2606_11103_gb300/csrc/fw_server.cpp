@@ -495,13 +495,13 @@ int fw_server_submit(fw_server *s, const fw_request *req, long long *id)
     const long long n_rec = (r.n_steps + r.decim - 1) / r.decim;
     // medium + upload staging (one dense map and the beta map at most) +
     // source and receiver buffers, each rounded to the arena's granule: per
-    // source its cell, gain, waveform row and partner (fw_set_sources) and its
-    // entry twice (the list grows when the receivers come: old and new one at
-    // once), per receiver its cell, partner, entry and traces
+    // source its cell, gain and waveform row and its entry twice (the list grows
+    // when the receivers come: old and new one at once), per receiver its entry
+    // and traces
     const size_t padded = (size_t)((r.grid.nx + 31) / 32 * 32) * r.grid.ny * r.grid.nz;
     const size_t entry = sizeof(fwgb::IoEntry);
-    j->footprint = bytes + padded * 8 + (size_t)n_src * (20 + 2 * entry) + (size_t)r.n_wave * r.n_steps * 8 +
-                   (size_t)n_rcv * (12 + entry + 4 * n_rec) + (16u << 20);
+    j->footprint = bytes + padded * 8 + (size_t)n_src * (16 + 2 * entry) + (size_t)r.n_wave * r.n_steps * 8 +
+                   (size_t)n_rcv * (entry + 4 * n_rec) + (16u << 20);
     std::lock_guard<std::mutex> lk(s->mu);
     j->id = s->next_id++;
     j->t_submit = s->now();
