@@ -371,9 +371,9 @@ int fw_load_state(fw_medium *m, const void *src, void *stream);
  * grad_alpha0 may be NULL.  Device memory: ceil(n_steps/K) + 2(K - 1) + 2
  * state images (about fw_state_bytes each), 2D + 1 fields, 4 FP64 maps and
  * the two output maps, from the installed allocator.  Without an installed
- * allocator they are kept for the medium's next gradient as long as those of
- * all media together take at most 8 GiB and a quarter of the device's free
- * memory, and given back by fw_release_workspace, fw_destroy_medium,
+ * allocator they are kept for the medium's next gradient if they take at most
+ * 8 GiB and those of all media together at most a quarter of the memory that
+ * the device has free beside them, and given back by fw_release_workspace, fw_destroy_medium,
  * fw_set_allocator and when an allocation of the library fails; an installed
  * allocator has them back before return.  The
  * recomputation of one segment runs on a stream of its own beside the

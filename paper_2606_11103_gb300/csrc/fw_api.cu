@@ -100,9 +100,9 @@ namespace fwgb {
 // ---- workspaces kept with their media -------------------------------------------
 // The last gradient's device buffers stay with the medium for its next gradient
 // (allocating and freeing the 4.2 GiB of a 1024^2 gradient of 128 steps took 4.4
-// of its 15.2 ms): those of all media together at most 8 GiB and a quarter of
-// what the device has free.  (Larger ones belong to longer gradients: 8.3 ms
-// for 14.4 GiB, 3000 steps at 1024^2, of 260 ms.)  Never from an allocator that the caller installed,
+// of its 15.2 ms): one of at most 8 GiB (larger ones belong to longer gradients:
+// 8.3 ms for 14.4 GiB, 3000 steps at 1024^2, of 260 ms), those of all media
+// together at most a quarter of what the device has free beside them.  Never from an allocator that the caller installed,
 // whose pool is the place to keep memory.  Idle ones are given back when an
 // allocation of the library fails, when an allocator is installed, on
 // fw_release_workspace and with the medium.
@@ -159,12 +159,12 @@ void workspace_give(fw_medium *m, void *p, size_t bytes)
         m->ws_busy = false;
         return;
     }
-    bool keep = !t_hook.alloc && !m->ws;
+    bool keep = !t_hook.alloc && !m->ws && bytes <= (8ULL << 30);
     {
         std::lock_guard<std::mutex> la(g_alloc_mu);
         keep = keep && !g_alloc;
     }
-    keep = keep && cudaMemGetInfo(&avail, &total) == cudaSuccess && g_ws_bytes + bytes <= std::min<size_t>(8ULL << 30, avail / 4);
+    keep = keep && cudaMemGetInfo(&avail, &total) == cudaSuccess && g_ws_bytes + bytes <= avail / 4;
     if (!keep) {
         lk.unlock();
         cudaGetLastError();
