@@ -415,7 +415,7 @@ __global__ void __launch_bounds__(AdjCta<R, DIM>::BX * AdjCta<R, DIM>::BY, sizeo
     prefetch(A.gs + P.i);
     // the pressure side's terms: in 2D they start the step's sum, in 3D (three
     // axes' terms more) the two sides add up in FP64 (128^3, N = 2: 9.58 ->
-    // 9.72 ms per gradient of 48 steps)
+    // 9.68 ms per gradient of 48 steps; loaded at the end 9.74)
     if (DIM == 3) {
         prefetch(A.gsp + P.i);
         gs[0] = gs[1] = gs[2] = gs[3] = R(0);
@@ -427,12 +427,12 @@ __global__ void __launch_bounds__(AdjCta<R, DIM>::BX * AdjCta<R, DIM>::BY, sizeo
         for (int e = 0; e < 4; ++e) rr[e] = adj_ramp(A, P, e);
     adj_velocity_axis<R, DIM, NM, 0>(A, P, cls, own, rr, gs);
     if (DIM == 3) adj_velocity_axis<R, DIM, NM, 1>(A, P, cls, own, rr, gs);
+    R gp[4];
+    if (DIM == 3) Io<R>::ld(A.gsp + P.i, gp);
     adj_velocity_axis<R, DIM, NM, 2>(A, P, cls, own, rr, gs);
     pdl_launch();
     double g[4] = {double(gs[0]), double(gs[1]), double(gs[2]), double(gs[3])};
     if (DIM == 3) {
-        R gp[4];
-        Io<R>::ld(A.gsp + P.i, gp);
 #pragma unroll
         for (int e = 0; e < 4; ++e) g[e] += double(gp[e]);
     }
