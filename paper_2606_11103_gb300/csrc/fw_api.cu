@@ -250,9 +250,9 @@ EncodeTiledFn tensor_map_encoder()
     return fn;
 }
 
-// Tensor maps of the 3D velocity sweep's streams; the sweep falls back to
-// per-thread cp.async staging where they cannot be built (or when the
-// environment sets FWGB_NO_TMA=1, for measurement).
+// Tensor maps of the sweeps' streams; where they cannot be built (or when the
+// environment sets FWGB_NO_TMA=1, for measurement) the 3D sweeps stage by
+// per-thread cp.async and the 2D ones read straight into registers.
 void setup_tma(fw_medium *m)
 {
     m->tma = false;

@@ -43,19 +43,19 @@ struct Monitor {
     int timeout;             // a bounded wait of a sweep on its staged copies gave up
 };
 
-// Tensor-map descriptors of the staged streams of the 3D velocity sweep
+// Tensor-map descriptors of the streams that a medium's velocity sweep stages
 // (opaque 128-byte driver objects, built on the host at medium creation):
-// p with its x/y halo box and p own box, v_d, psi1[m][d], rho with its +1
-// halo box and rho own box, the class index and K dt.
+// p with its halo box and (3D) p own box, v_d, psi1[m][d], rho with its +1
+// halo box and (3D) rho own box, the class index and K dt.
 struct alignas(64) TensorMapBlob {
     unsigned char bytes[128];
 };
 struct VelMaps {
     TensorMapBlob p_halo, p_own, v[3], psi[FW_MAX_MECH][3], rho_halo, rho_own, cls, kdt;
 };
-// ... and of the 3D pressure sweep: v_z own box (planes ahead), v_x with its
-// x halo, v_y with its y halo, p, K dt, 2 beta dt, psi2[m], the class index,
-// rho (time-space stencil)
+// ... and its pressure sweep: v_z own box (3D: planes ahead; 2D: with its halo
+// rows), v_x with its x halo, v_y with its y halo (3D), p, K dt, 2 beta dt,
+// psi2[m], the class index, rho (time-space stencil)
 struct PresMaps {
     TensorMapBlob vz_own, vx_halo, vy_halo, p_own, kdt, b2dt, psi[FW_MAX_MECH], cls, rho_own;
     TensorMapBlob vx_ring, vy_ring, vz_ring;   // time-space stencil: v boxes with x and y halos
@@ -158,7 +158,7 @@ struct fw_medium {
     double psi_pref = 10.0;          // pressure reference [Pa] of binary16 memory variables
     int time_order = 2;              // 2: leapfrog; 4: time-space stencil (Sec. 3.3)
     double ts_a[4][4] = {};          // time-space weights a_m = sum_n ts_a[m][n] r^(2n)
-    bool tma = false;                // 3D sweeps staged by tensor-memory-access copies
+    bool tma = false;                // the tensor maps below are there: sweeps staged by TMA copies
     fwgb::VelMaps vel_maps{};
     fwgb::PresMaps pres_maps{};
 };

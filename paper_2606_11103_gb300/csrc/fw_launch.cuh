@@ -252,10 +252,16 @@ PresArgs<R, SS, SP> pres_args(const fw_medium *m, const StepImages *im, const St
 // (StepImages) instead of the in-place step of the medium's own state.
 // 2D FP32-state grids from kTileMin tiles on take the staged sweeps, in runs of
 // two tiles per CTA, of four from kTileLong tiles on; smaller grids, FP64 media
-// and image steps the unstaged ones.  Measured, us per step (unstaged / staged
-// in runs of 1, 2, 4, 8; N = 4, FP32): 512^2 (512 tiles) 10.7 / 13.1, 13.9,
-// 20.1, 32.3; 1024^2 (2048) 28.3 / 30.7, 27.6, 31.5, 38.9; 2048^2 (8192) 116 /
-// 114, 102, 104, 110; 4096^2 (32768) 431 / 415, 373, 363, 373.  A run hides
+// and image steps the unstaged ones.  Measured when the line was drawn, us per
+// step (unstaged / staged in runs of 1, 2, 4, 8; N = 4, FP32): 512^2 (512 tiles)
+// 10.7 / 13.1, 13.9, 20.1, 32.3; 1024^2 (2048) 28.3 / 30.7, 27.6, 31.5, 38.9;
+// 2048^2 (8192) 116 / 114, 102, 104, 110; 4096^2 (32768) 431 / 415, 373, 363, 373.
+// With sources inside the sweeps and programmatic launch (unstaged / staged;
+// FP32 N = 2, N = 4, bfloat16 N = 4, time-space N = 4): 1024^2 19.8 / 21.7, 24.9 /
+// 27.1, 20.8 / 23.4, 34.8 / 33.2; 1456^2 (4368) 38.7 / 38.3, 56.1 / 55.1, 41.8 /
+// 41.9, 73.1 / 63.4; 2048^2 83.3 / 74.2, 112 / 102, 87.2 / 77.9, 142 / 115;
+// 4096^2 316 / 253, 427 / 367, 330 / 262, 536 / 395: the leapfrog's two forms meet
+// at about 4400 tiles now, the time-space stencil's at 2048.  A run hides
 // the latency of a tile's copies behind the tile before it, a short one leaves
 // the hardware more CTAs to balance: with one persistent CTA per slot and even
 // shares the 4096^2 step took 439 us, its slowest SMs finishing last.

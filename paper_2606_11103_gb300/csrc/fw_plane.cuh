@@ -1,7 +1,7 @@
 // Sweeps of 2D grids (kernel axes x and depth): one thread per quad of four
 // consecutive x points, no march along the depth (the 3D sweeps' form).  A
 // marching CTA walks its rows one after the other: on a 256^2 grid 32 CTAs of
-// 64 threads did all the work (27 us per step, 8.1 us now).
+// 64 threads did all the work (27 us per step, 6.3 us now).
 //
 // Small grids (k_velocity_plane, k_pressure_plane): bound by launches and by
 // the latency of one pass of loads, so every stream is read straight into
